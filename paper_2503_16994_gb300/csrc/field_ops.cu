@@ -242,20 +242,21 @@ __global__ void __launch_bounds__(64) clover_build_kernel(Geom g, LinkField<F64>
     int x[4];
     cb_coords(g, p, cb, x);
     const bool open = bc == LQCD_BC_OPEN, sf = bc == LQCD_BC_SF;
-    m3 Fxy = field_strength(g, U, x, 0, 1, open), Fxz = field_strength(g, U, x, 0, 2, open);
-    m3 Fxt = field_strength(g, U, x, 0, 3, open), Fyz = field_strength(g, U, x, 1, 2, open);
-    m3 Fyt = field_strength(g, U, x, 1, 3, open), Fzt = field_strength(g, U, x, 2, 3, open);
+    double plaq;
+    const ah3 Fxy = field_strength(g, U, x, 0, 1, open, plaq), Fxz = field_strength(g, U, x, 0, 2, open, plaq);
+    const ah3 Fxt = field_strength(g, U, x, 0, 3, open, plaq), Fyz = field_strength(g, U, x, 1, 2, open, plaq);
+    const ah3 Fyt = field_strength(g, U, x, 1, 3, open, plaq), Fzt = field_strength(g, U, x, 2, 3, open, plaq);
     const bool improved = open ? (x[3] == 0 || x[3] == g.L[3] - 1) : (sf && (x[3] == 1 || x[3] == g.L[3] - 1));
     const double diag = improved ? 1.0 + cfterm : 1.0;
     if (sf && x[3] == 0) kc = 0.0;  // the boundary slice: identity site term
     for (int blk = 0; blk < 2; ++blk) {
         const double sg = blk == 0 ? 1.0 : -1.0;
         cd A[6][6], Ai[6][6];
+        const m3 fx = ah_full(ah_axpy(sg, Fxt, 1.0, Fyz)), fy = ah_full(ah_axpy(sg, Fyt, -1.0, Fxz));
+        const m3 fz = ah_full(ah_axpy(sg, Fzt, 1.0, Fxy));
         for (int i = 0; i < 3; ++i)
             for (int j = 0; j < 3; ++j) {
-                cd Mx = Fyz.m[i][j] + sg * Fxt.m[i][j];
-                cd My = (-1.0) * Fxz.m[i][j] + sg * Fyt.m[i][j];
-                cd Mz = Fxy.m[i][j] + sg * Fzt.m[i][j];
+                const cd Mx = fx.m[i][j], My = fy.m[i][j], Mz = fz.m[i][j];
                 cd id = cd{i == j ? diag : 0.0, 0.0};
                 A[i][j] = id - kc * mul_i(Mz);
                 A[3 + i][3 + j] = id + kc * mul_i(Mz);

@@ -33,110 +33,264 @@ __device__ __forceinline__ void store_m3(double2 *base, long stride, long cb, co
     for (int k = 0; k < 9; ++k) base[k * stride + cb] = make_double2(m.m[k / 3][k % 3].re, m.m[k / 3][k % 3].im);
 }
 
-__device__ __forceinline__ m3 madd(const m3 &a, const m3 &b)
+// The antihermitian part of a stored matrix (fields that are antihermitian by
+// construction: the flow's accumulator X, the HMC momenta)
+__device__ __forceinline__ ah3 load_ah(const double2 *base, long stride, long cb)
 {
-    m3 r;
+    ah3 r;
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) r.m[i][j] = a.m[i][j] + b.m[i][j];
+    for (int i = 0; i < 3; ++i) r.d[i] = base[4 * i * stride + cb].y;
+    const double2 a = base[stride + cb], b = base[2 * stride + cb], c = base[5 * stride + cb];
+    r.o[0] = cd{a.x, a.y};
+    r.o[1] = cd{b.x, b.y};
+    r.o[2] = cd{c.x, c.y};
     return r;
 }
 
-__device__ m3 flow_generator(const Geom &g, const LinkField<F64> &U, const int x[4], int mu)
+// exp(s X) for antihermitian traceless X, as q0 + q1 Y + q2 Y^2 with Y = s X /
+// 2^k (Cayley-Hamilton: Y^3 = c1 Y + i c0 with c1 = tr Y^2 / 2 and i c0 =
+// det Y, both from Y and Y^2).  The three coefficients come from the Horner
+// form of the degree-20 Taylor polynomial, P <- 1/n! + Y P, which costs four
+// real operations a step instead of a 3x3 product, and the k squarings act on
+// the coefficients too.  k is chosen so that |Y|_F <= 1/2, where the terms
+// left out are below 1e-25.  About 200 FP64 instructions; a Taylor polynomial
+// with 3x3 products took 2900, and 22.4 ms for the links of 32^4 where
+// force_gather_kernel now takes 3.6 ms for the whole update.
+constexpr int kExpDegree = 20;
+__device__ __forceinline__ m3 exp_ah(const ah3 &X, double s)
 {
+    ah3 Y;
+    double n2 = 0.0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        Y.d[i] = s * X.d[i];
+        Y.o[i] = s * X.o[i];
+        n2 = fma(Y.d[i], Y.d[i], n2);
+        n2 = fma(2.0 * Y.o[i].re, Y.o[i].re, n2);
+        n2 = fma(2.0 * Y.o[i].im, Y.o[i].im, n2);
+    }
+    int k = 0;
+    double sc = 1.0;
+    while (n2 > 0.25 && k < 60) {
+        n2 *= 0.25;
+        sc *= 0.5;
+        ++k;
+    }
+    if (k > 0) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            Y.d[i] *= sc;
+            Y.o[i] = sc * Y.o[i];
+        }
+    }
+    // H = Y^2 (Hermitian): with Y = (i d0, a, b; -a*, i d1, c; -b*, -c*, i d2)
+    const cd a = Y.o[0], b = Y.o[1], c = Y.o[2];
+    const double na = fma(a.re, a.re, a.im * a.im), nb = fma(b.re, b.re, b.im * b.im), nc = fma(c.re, c.re, c.im * c.im);
+    const double h0 = -fma(Y.d[0], Y.d[0], na + nb), h1 = -fma(Y.d[1], Y.d[1], na + nc),
+                 h2 = -fma(Y.d[2], Y.d[2], nb + nc);
+    // H01 = i (d0 + d1) a - b c*, H02 = i (d0 + d2) b + a c, H12 = i (d1 + d2) c - a* b
+    const double s01 = Y.d[0] + Y.d[1], s02 = Y.d[0] + Y.d[2], s12 = Y.d[1] + Y.d[2];
+    cd ha = cd{-s01 * a.im, s01 * a.re}, hb = cd{-s02 * b.im, s02 * b.re}, hc = cd{-s12 * c.im, s12 * c.re};
+    cma(ha, cd{-b.re, -b.im}, cd{c.re, -c.im});
+    cma(hb, a, c);
+    cma(hc, cd{-a.re, a.im}, b);
+    const double c1 = 0.5 * (h0 + h1 + h2);
+    // i c0 = tr(Y^3) / 3: tr(H Y) = i (sum_i h_i d_i + 2 sum_(i<j) Im(H_ij* Y_ij))
+    double im = 0.0;
+    im = fma(ha.re, a.im, im);
+    im = fma(-ha.im, a.re, im);
+    im = fma(hb.re, b.im, im);
+    im = fma(-hb.im, b.re, im);
+    im = fma(hc.re, c.im, im);
+    im = fma(-hc.im, c.re, im);
+    const double c0 = (1.0 / 3.0) * fma(h0, Y.d[0], fma(h1, Y.d[1], fma(h2, Y.d[2], 2.0 * im)));
+    // Horner: (q0, q1, q2) <- (1/n! + i c0 q2, q0 + c1 q2, q1)
+    double f[kExpDegree + 1];
+    f[0] = 1.0;
+#pragma unroll
+    for (int n = 1; n <= kExpDegree; ++n) f[n] = f[n - 1] / n;
+    cd q0 = cd{f[kExpDegree], 0.0}, q1 = cd{0.0, 0.0}, q2 = cd{0.0, 0.0};
+#pragma unroll
+    for (int n = kExpDegree - 1; n >= 0; --n) {
+        const cd t0 = cd{fma(-c0, q2.im, f[n]), c0 * q2.re};
+        const cd t1 = cd{fma(c1, q2.re, q0.re), fma(c1, q2.im, q0.im)};
+        q2 = q1;
+        q1 = t1;
+        q0 = t0;
+    }
+    // squarings: Y^3 = c1 Y + i c0, Y^4 = c1 Y^2 + i c0 Y
+    for (int n = 0; n < k; ++n) {
+        const cd p12 = 2.0 * cm0(q1, q2), p22 = cm0(q2, q2);
+        cd t0 = cd{-c0 * p12.im, c0 * p12.re};
+        cma(t0, q0, q0);
+        cd t1 = cd{fma(c1, p12.re, -c0 * p22.im), fma(c1, p12.im, c0 * p22.re)};
+        cma(t1, 2.0 * q0, q1);
+        cd t2 = c1 * p22;
+        cma(t2, q1, q1);
+        cma(t2, 2.0 * q0, q2);
+        q0 = t0;
+        q1 = t1;
+        q2 = t2;
+    }
+    m3 E;
+    const double h[3] = {h0, h1, h2};
+    const cd hh[3] = {ha, hb, hc};
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+        E.m[i][i] = cd{fma(q2.re, h[i], fma(-q1.im, Y.d[i], q0.re)), fma(q2.im, h[i], fma(q1.re, Y.d[i], q0.im))};
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        const int i = e == 2 ? 1 : 0, j = e == 0 ? 1 : 2;
+        cd u = cm0(q1, Y.o[e]);
+        cma(u, q2, hh[e]);
+        E.m[i][j] = u;
+        cd l = cm0(q1, cd{-Y.o[e].re, Y.o[e].im});
+        cma(l, q2, cd{hh[e].re, -hh[e].im});
+        E.m[j][i] = l;
+    }
+    return E;
+}
+
+__device__ __forceinline__ ah3 ah_sum(const ah3 &a, double s, const ah3 &b)
+{
+    return ah_axpy(1.0, a, s, b);
+}
+
+// ---------------------------------------------------------------------------
+// Links and force.  Every plaquette P = B1 B2^dag with B1 = U_mu(x) U_nu(x+mu)
+// and B2 = U_nu(x) U_mu(x+nu) serves four links: the two at x take P - P^dag
+// (with opposite signs), and B1^dag U_nu(x), B2^dag U_mu(x) are the lower
+// staples of U_mu(x+nu) and U_nu(x+mu).  One thread per (site, plane) forms
+// them once (6 planes x 522 FP64 instructions a site), and one thread per link
+// adds its three upper and three lower terms (about 200 with the link's
+// product): 3900 instructions a site against 5700 for the six staples of each
+// link formed separately.  The kernels are bound by the FP64 pipe (89% busy),
+// so the instructions decide: on 32^4 plaquette_kernel takes 5.5 ms and
+// force_gather_kernel, which also updates the link, 3.6 ms, where the staples
+// per link and the update took 15.4 and 22.4 ms (six instructions per complex
+// product, the exponential by 3x3 products).  It costs scratch (FlowScratch,
+// 2160 bytes a site); where the device has no room for that,
+// flow_force_kernel forms the staples (10.7 ms, and 2.3 ms for the update).
+// ---------------------------------------------------------------------------
+struct FlowScratch {
+    double2 *low = nullptr;  // lower staples [parity][mu][slot of nu][9 planes]
+    double *up = nullptr;    // P - P^dag [parity][plane][9 planes]: diagonal (imaginary), then the 3 upper entries
+    static size_t low_bytes(long stride) { return sizeof(double2) * 2 * 4 * 3 * 9 * (size_t)stride; }
+    static size_t up_bytes(long stride) { return sizeof(double) * 2 * 6 * 9 * (size_t)stride; }
+};
+
+// planes (0,1) (0,2) (0,3) (1,2) (1,3) (2,3)
+__device__ __forceinline__ int plane_of(int mu, int nu)  // mu < nu
+{
+    return mu == 0 ? nu - 1 : (mu == 1 ? nu + 1 : 5);
+}
+
+__global__ void __launch_bounds__(128) plaquette_kernel(Geom g, LinkField<F64> U, double2 *low, double *up)
+{
+    const int cb = blockIdx.x * blockDim.x + threadIdx.x;
+    const int p = blockIdx.y, plane = blockIdx.z;
+    if (cb >= g.vh) return;
+    const int mu = plane < 3 ? 0 : (plane < 5 ? 1 : 2), nu = plane < 3 ? plane + 1 : (plane < 5 ? plane - 1 : 3);
+    int x[4];
+    cb_coords(g, p, cb, x);
+    const int ym = cb_neighbour(g, x, mu, +1), yn = cb_neighbour(g, x, nu, +1);
+    const m3 Um = load_link<F64, double>(U, p, mu, cb), Un = load_link<F64, double>(U, p, nu, cb);
+    const m3 B1 = mm(Um, load_link<F64, double>(U, p ^ 1, nu, ym));
+    const m3 B2 = md(mm(Un, load_link<F64, double>(U, p ^ 1, mu, yn)));
+    ah3 w = ah_zero();
+    ah_add(w, B1, B2);
+    double *u = up + (long)(p * 6 + plane) * 9 * g.stride + cb;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        u[i * g.stride] = w.d[i];
+        u[(3 + 2 * i) * g.stride] = w.o[i].re;
+        u[(4 + 2 * i) * g.stride] = w.o[i].im;
+    }
+    // slot of direction b among the three others of a: b < a ? b : b - 1
+    store_m3(low + (long)(((p ^ 1) * 4 + mu) * 3 + nu - 1) * 9 * g.stride, g.stride, yn, mm(md(B1), Un));
+    store_m3(low + (long)(((p ^ 1) * 4 + nu) * 3 + mu) * 9 * g.stride, g.stride, ym, mm(B2, Um));
+}
+
+// X <- a Z + b X, and the link U <- exp(s X) U when s != 0, for the
+// antihermitian om = Omega - Omega^dag (Z = -om / 2 without its trace)
+__device__ __forceinline__ void force_finish(const ah3 &om, const m3 &u, double2 *X, double2 *ub, long stride, long cb,
+                                             double a, double b, double s)
+{
+    ah3 x = ah_traceless(om, -0.5 * a);
+    if (b != 0.0) x = ah_sum(x, b, load_ah(X, stride, cb));
+    store_m3(X, stride, cb, ah_full(x));
+    if (s != 0.0) store_m3(ub, stride, cb, mm(exp_ah(x, s), u));
+}
+
+__global__ void __launch_bounds__(128) force_gather_kernel(Geom g, double2 *u64, const double2 *low, const double *up,
+                                                           double2 *X, double a, double b, double s)
+{
+    const long cb = long(blockIdx.x) * blockDim.x + threadIdx.x;
+    const int p = blockIdx.y, mu = blockIdx.z;
+    if (cb >= g.vh) return;
+    const long q = p * 4 + mu;
+    m3 S = load_m3(low + q * 27 * g.stride, g.stride, cb);
+#pragma unroll
+    for (int n = 1; n < 3; ++n) {
+        const m3 t = load_m3(low + (q * 3 + n) * 9 * g.stride, g.stride, cb);
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) S.m[i][j] = S.m[i][j] + t.m[i][j];
+    }
+    double2 *ub = u64 + q * 9 * g.stride;
+    const m3 u = load_m3(ub, g.stride, cb);
+    ah3 om = ah_zero();
+    ah_add(om, u, S);
+#pragma unroll
+    for (int n = 0; n < 3; ++n) {
+        const int nu = n < mu ? n : n + 1;
+        const double sg = nu > mu ? 1.0 : -1.0;
+        const double *w = up + (long)(p * 6 + (nu > mu ? plane_of(mu, nu) : plane_of(nu, mu))) * 9 * g.stride + cb;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            om.d[i] = fma(sg, w[i * g.stride], om.d[i]);
+            om.o[i].re = fma(sg, w[(3 + 2 * i) * g.stride], om.o[i].re);
+            om.o[i].im = fma(sg, w[(4 + 2 * i) * g.stride], om.o[i].im);
+        }
+    }
+    force_finish(om, u, X + q * 9 * g.stride, ub, g.stride, cb, a, b, s);
+}
+
+// X_mu(x) = a Z_mu(x) + b X_mu(x) for every link (b = 0: X not read), the
+// staples formed here: no scratch
+__global__ void __launch_bounds__(64) flow_force_kernel(Geom g, LinkField<F64> U, double2 *X, double a, double b)
+{
+    const long cb = long(blockIdx.x) * blockDim.x + threadIdx.x;
+    const int p = blockIdx.y, mu = blockIdx.z;
+    if (cb >= g.vh) return;
+    int x[4], xpm[4];
+    cb_coords(g, p, int(cb), x);
+    shift(g, x, mu, +1, xpm);
     m3 S;
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int j = 0; j < 3; ++j) S.m[i][j] = cd{0.0, 0.0};
-    int xpm[4];
-    shift(g, x, mu, +1, xpm);
     for (int nu = 0; nu < 4; ++nu) {
         if (nu == mu) continue;
         int xpn[4], xmn[4], xpm_mn[4];
         shift(g, x, nu, +1, xpn);
         shift(g, x, nu, -1, xmn);
         shift(g, xpm, nu, -1, xpm_mn);
-        S = madd(S, mm(mm(link_xy(g, U, xpm, nu, false), md(link_xy(g, U, xpn, mu, false))),
-                       md(link_xy(g, U, x, nu, false))));
-        S = madd(S, mm(mm(md(link_xy(g, U, xpm_mn, nu, false)), md(link_xy(g, U, xmn, mu, false))),
-                       link_xy(g, U, xmn, nu, false)));
-    }
-    const m3 om = mm(link_xy(g, U, x, mu, false), S);
-    m3 Z;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) Z.m[i][j] = -0.5 * (om.m[i][j] - conj(om.m[j][i]));
-    const cd tr = (1.0 / 3.0) * (Z.m[0][0] + Z.m[1][1] + Z.m[2][2]);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) Z.m[i][i] = Z.m[i][i] - tr;
-    return Z;
-}
-
-// X_mu(x) = a Z_mu(x) + b X_mu(x) for every link (b = 0: X not read)
-__global__ void __launch_bounds__(64) flow_force_kernel(Geom g, LinkField<F64> U, double2 *X, double a, double b)
-{
-    const long cb = long(blockIdx.x) * blockDim.x + threadIdx.x;
-    const int p = blockIdx.y, mu = blockIdx.z;
-    if (cb >= g.vh) return;
-    int x[4];
-    cb_coords(g, p, int(cb), x);
-    const m3 Z = flow_generator(g, U, x, mu);
-    double2 *xb = X + (long)(p * 4 + mu) * 9 * g.stride;
-    m3 r;
-    if (b != 0.0) {
-        const m3 old = load_m3(xb, g.stride, cb);
+        const m3 f = mm(mm(link_xy(g, U, xpm, nu, false), md(link_xy(g, U, xpn, mu, false))),
+                        md(link_xy(g, U, x, nu, false)));
+        const m3 r = mm(mm(md(link_xy(g, U, xpm_mn, nu, false)), md(link_xy(g, U, xmn, mu, false))),
+                        link_xy(g, U, xmn, nu, false));
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
-            for (int j = 0; j < 3; ++j) r.m[i][j] = a * Z.m[i][j] + b * old.m[i][j];
-    } else {
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) r.m[i][j] = a * Z.m[i][j];
+            for (int j = 0; j < 3; ++j) S.m[i][j] = S.m[i][j] + f.m[i][j] + r.m[i][j];
     }
-    store_m3(xb, g.stride, cb, r);
-}
-
-// exp(X) by scaling and squaring of a degree-16 Taylor polynomial (Horner
-// form): X / 2^s has a row-sum norm <= 1/4, where the truncated terms are
-// below 1e-25 of the sum
-__device__ m3 expm3(const m3 &X)
-{
-    double n = 0.0;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        double r = 0.0;
-#pragma unroll
-        for (int j = 0; j < 3; ++j) r += sqrt(norm2(X.m[i][j]));
-        n = fmax(n, r);
-    }
-    int s = 0;
-    while (n > 0.25 && s < 60) {
-        n *= 0.5;
-        ++s;
-    }
-    const double sc = ldexp(1.0, -s);
-    m3 Y, E;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            Y.m[i][j] = sc * X.m[i][j];
-            E.m[i][j] = cd{i == j ? 1.0 : 0.0, 0.0};
-        }
-    for (int k = 16; k >= 1; --k) {  // E = 1 + Y E / k
-        const m3 YE = mm(Y, E);
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) E.m[i][j] = cd{i == j ? 1.0 : 0.0, 0.0} + (1.0 / k) * YE.m[i][j];
-    }
-    for (int k = 0; k < s; ++k) E = mm(E, E);
-    return E;
+    const m3 u = link_xy(g, U, x, mu, false);
+    ah3 om = ah_zero();
+    ah_add(om, u, S);
+    force_finish(om, u, X + (long)(p * 4 + mu) * 9 * g.stride, nullptr, g.stride, cb, a, b, 0.0);
 }
 
 // U_mu(x) <- exp(s X_mu(x)) U_mu(x)
@@ -146,14 +300,8 @@ __global__ void __launch_bounds__(128) flow_update_kernel(Geom g, double2 *u64, 
     const int p = blockIdx.y, mu = blockIdx.z;
     if (cb >= g.vh) return;
     double2 *ub = u64 + (long)(p * 4 + mu) * 9 * g.stride;
-    const double2 *xb = X + (long)(p * 4 + mu) * 9 * g.stride;
-    m3 x = load_m3(xb, g.stride, cb);
-    if (s != 1.0)
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) x.m[i][j] = s * x.m[i][j];
-    store_m3(ub, g.stride, cb, mm(expm3(x), load_m3(ub, g.stride, cb)));
+    const ah3 x = load_ah(X + (long)(p * 4 + mu) * 9 * g.stride, g.stride, cb);
+    store_m3(ub, g.stride, cb, mm(exp_ah(x, s), load_m3(ub, g.stride, cb)));
 }
 
 // HMC momenta: P_mu(x) = sum_a pi_a i lambda_a / 2 from the caller's
@@ -269,25 +417,17 @@ __global__ void __launch_bounds__(128) gauge_obs_kernel(Geom g, LinkField<F64> U
         x[1] = int(r % g.L[1]);
         x[2] = int(r / g.L[1]);
         x[3] = t;
-        const int planes[6][2] = {{0, 1}, {0, 2}, {0, 3}, {1, 2}, {1, 3}, {2, 3}};
-        m3 F[6];
+        ah3 F[6];
+#pragma unroll
         for (int q = 0; q < 6; ++q) {
-            const int mu = planes[q][0], nu = planes[q][1];
-            int xpm[4], xpn[4];
-            shift(g, x, mu, +1, xpm);
-            shift(g, x, nu, +1, xpn);
-            const m3 P = mm(mm(link_xy(g, U, x, mu, false), link_xy(g, U, xpm, nu, false)),
-                            mm(md(link_xy(g, U, xpn, mu, false)), md(link_xy(g, U, x, nu, false))));
-            const double re = P.m[0][0].re + P.m[1][1].re + P.m[2][2].re;
+            const int mu = q < 3 ? 0 : (q < 5 ? 1 : 2), nu = q < 3 ? q + 1 : (q < 5 ? q - 1 : 3);
+            double re;
+            F[q] = field_strength(g, U, x, mu, nu, false, re);
             v[0] += re / 3.0;
             v[1] += 2.0 * (3.0 - re);
-            F[q] = field_strength(g, U, x, mu, nu, false);
-            const m3 FF = mm(F[q], F[q]);
-            v[2] -= FF.m[0][0].re + FF.m[1][1].re + FF.m[2][2].re;
+            v[2] -= ah_tr(F[q], F[q]);
         }
-        const m3 a = mm(F[0], F[5]), b = mm(F[1], F[4]), d = mm(F[2], F[3]);
-        const double e = (a.m[0][0].re + a.m[1][1].re + a.m[2][2].re) - (b.m[0][0].re + b.m[1][1].re + b.m[2][2].re) +
-                         (d.m[0][0].re + d.m[1][1].re + d.m[2][2].re);
+        const double e = ah_tr(F[0], F[5]) - ah_tr(F[1], F[4]) + ah_tr(F[2], F[3]);
         v[3] = -8.0 * e / (32.0 * 3.14159265358979323846 * 3.14159265358979323846);
     }
     for (int o = 0; o < 4; ++o)
@@ -319,24 +459,64 @@ __global__ void __launch_bounds__(128) gauge_unpack_kernel(Geom g, long V, const
     }
 }
 
-// one stage of the low-storage RK3 step (W_stage -> W_stage+1) of the links
-// u (FP64 planes), X the stage accumulator
-static void flow_stage(lqcd_lattice_s *lat, double2 *u, double2 *X, int stage, double eps, cudaStream_t st)
+// scratch of the shared-plaquette force for one call; empty (both pointers
+// null) when the device has no room for it
+struct FlowWork {
+    DevBuf low, up;
+    FlowScratch s;
+    explicit FlowWork(long stride)
+    {
+        try {
+            low.ensure(FlowScratch::low_bytes(stride));
+            up.ensure(FlowScratch::up_bytes(stride));
+            s = FlowScratch{low.as<double2>(), up.as<double>()};
+        } catch (const Error &e) {
+            if (e.code != LQCD_ENOMEM) throw;
+            cudaGetLastError();  // the failed allocation is not an error of the call
+            low.release();
+            up.release();
+        }
+    }
+};
+
+// X <- a Z(u) + b X, then u <- exp(s X) u (s = 0: the force only)
+static void force_step(lqcd_lattice_s *lat, double2 *u, double2 *X, const FlowScratch &w, double a, double b, double s,
+                       const char *force_name, const char *update_name, cudaStream_t st)
 {
     const long S = lat->stride;
-    const dim3 gf(unsigned((lat->vh + 63) / 64), 2, 4), gu(unsigned((lat->vh + 127) / 128), 2, 4);
-    // per link: 6 staples of 2 products and a product with the link (~13 3x3 complex products)
-    const double fbytes = double(lat->V) * 4 * (7 * 144.0 + 144.0), ubytes = double(lat->V) * 4 * 3 * 144.0;
     const LinkField<F64> U{u, nullptr, S};
-    const double a[3] = {0.25, 8.0 / 9.0, 0.75}, b[3] = {0.0, -17.0 / 9.0, -1.0};
+    const unsigned nb = unsigned((lat->vh + 127) / 128);
+    if (w.low) {
+        {
+            // reads the 4 links of a site, writes 12 staples and 6 antihermitian matrices
+            ProfScope prof(force_name, double(lat->V) * (4 * 144.0 + 12 * 144.0 + 6 * 72.0), st);
+            plaquette_kernel<<<dim3(nb, 2, 6), 128, 0, st>>>(lat->geom, U, w.low, w.up);
+            LQCD_CHECK_LAUNCH();
+        }
+        ProfScope prof(update_name, double(lat->V) * 4 * (3 * 144.0 + 3 * 72.0 + 4 * 144.0), st);
+        force_gather_kernel<<<dim3(nb, 2, 4), 128, 0, st>>>(lat->geom, u, w.low, w.up, X, a, b, s);
+        LQCD_CHECK_LAUNCH();
+        return;
+    }
     {
-        ProfScope prof("flow_force", fbytes, st);
-        flow_force_kernel<<<gf, 64, 0, st>>>(lat->geom, U, X, a[stage] * eps, b[stage]);
+        ProfScope prof(force_name, double(lat->V) * 4 * (7 * 144.0 + 144.0), st);
+        flow_force_kernel<<<dim3(unsigned((lat->vh + 63) / 64), 2, 4), 64, 0, st>>>(lat->geom, U, X, a, b);
         LQCD_CHECK_LAUNCH();
     }
-    ProfScope prof("flow_update", ubytes, st);
-    flow_update_kernel<<<gu, 128, 0, st>>>(lat->geom, u, X, 1.0);
-    LQCD_CHECK_LAUNCH();
+    if (s != 0.0) {
+        ProfScope prof(update_name, double(lat->V) * 4 * 3 * 144.0, st);
+        flow_update_kernel<<<dim3(nb, 2, 4), 128, 0, st>>>(lat->geom, u, X, s);
+        LQCD_CHECK_LAUNCH();
+    }
+}
+
+// one stage of the low-storage RK3 step (W_stage -> W_stage+1) of the links
+// u (FP64 planes), X the stage accumulator
+static void flow_stage(lqcd_lattice_s *lat, double2 *u, double2 *X, const FlowScratch &w, int stage, double eps,
+                       cudaStream_t st)
+{
+    const double a[3] = {0.25, 8.0 / 9.0, 0.75}, b[3] = {0.0, -17.0 / 9.0, -1.0};
+    force_step(lat, u, X, w, a[stage] * eps, b[stage], 1.0, "flow_force", "flow_update", st);
 }
 
 // the FP32/FP16 copies of the flowed links; the clover fields of the old links are dropped
@@ -356,8 +536,10 @@ void gauge_flow(lqcd_lattice_s *lat, GaugeSet &g, double eps, int nsteps, cudaSt
     const long S = lat->stride;
     DevBuf X;
     X.ensure(sizeof(double2) * 2 * 4 * 9 * S);
+    const FlowWork w(S);
     for (int k = 0; k < nsteps; ++k)
-        for (int stage = 0; stage < 3; ++stage) flow_stage(lat, g.u64.as<double2>(), X.as<double2>(), stage, eps, st);
+        for (int stage = 0; stage < 3; ++stage)
+            flow_stage(lat, g.u64.as<double2>(), X.as<double2>(), w.s, stage, eps, st);
     flow_finish(lat, g, st);
 }
 
@@ -378,66 +560,101 @@ void gauge_flow(lqcd_lattice_s *lat, GaugeSet &g, double eps, int nsteps, cudaSt
 // ---------------------------------------------------------------------------
 struct Phases {
     double re[4], im[4];
+    int mask;  // bit mu set: the phase of direction mu is not 1
 };
 
-__global__ void __launch_bounds__(128) laplace_kernel(Geom g, int p, LinkField<F64> U, Phases th,
-                                                      SpinorField<F64> self, SpinorField<F64> other,
-                                                      SpinorField<F64> a1, SpinorField<F64> a2, SpinorField<F64> out,
-                                                      int nrhs, double cH, double c0, double c1, double c2)
+static Phases phases_of(const lqcd_dirac_params &dp)
 {
+    Phases th;
+    hop_theta(dp, th.re, th.im);
+    th.mask = 0;
+    for (int mu = 0; mu < 4; ++mu)
+        if (th.re[mu] != 1.0 || th.im[mu] != 0.0) th.mask |= 1 << mu;
+    return th;
+}
+
+// a field by its two parity halves
+struct Halves {
+    SpinorField<F64> h[2];
+};
+
+// acc += W v on the colour index of all four spins, W = U or U^dag, with the
+// boundary phase applied to v where the hop wraps: 144 FP64 instructions (the
+// sums run inside the products' fma chains)
+template <bool DAG>
+__device__ __forceinline__ void colour_hop(spinor<double> &acc, const su3<double> &u, spinor<double> v, bool wrap,
+                                           double ph_re, double ph_im)
+{
+    if (wrap) {
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) v.s[s][a] = cm0(cd{ph_re, ph_im}, v.s[s][a]);
+    }
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b)
+                cma(acc.s[s][a], DAG ? cd{u.m[b][a].re, -u.m[b][a].im} : u.m[a][b], v.s[s][b]);
+}
+
+// One thread per (site, right-hand side), both parities in one launch
+// (blockIdx.y).  Bound by the FP64 pipe: 1152 instructions for the eight hops
+// and 24 to 72 for the sums with in, a1 and a2; phases cost only where a hop
+// wraps under a phase other than 1.  3.14 ms for twelve fields on 16^3 x 32,
+// against 6.2 ms with separate products and sums and a phase on every hop.
+__global__ void __launch_bounds__(128) laplace_kernel(Geom g, LinkField<F64> U, Phases th, Halves in, Halves a1,
+                                                      Halves a2, Halves out, int nrhs, double cH, double c0, double c1,
+                                                      double c2)
+{
+    const int p = blockIdx.y;
     const int j = blockIdx.x % nrhs, tile = blockIdx.x / nrhs;
     const int cb = tile * blockDim.x + threadIdx.x;
     if (cb >= g.vh) return;
     int x[4];
     cb_coords(g, p, cb, x);
+    const SpinorField<F64> other = p ? in.h[0] : in.h[1];
     spinor<double> acc;
     zero(acc);
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
-        int y[4];
-        shift(g, x, mu, +1, y);
-        int ycb = cb_index(g, y);
-        const su3<double> Uf = load_link<F64, double>(U, p, mu, cb);
-        spinor<double> v = load_spinor<F64, double>(other, j, ycb);
-        cx<double> ph = x[mu] == g.L[mu] - 1 ? cx<double>{th.re[mu], th.im[mu]} : cx<double>{1.0, 0.0};
-#pragma unroll
-        for (int s = 0; s < 4; ++s)
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-                acc.s[s][a] = acc.s[s][a] + ph * (Uf.m[a][0] * v.s[s][0] + Uf.m[a][1] * v.s[s][1] + Uf.m[a][2] * v.s[s][2]);
-        shift(g, x, mu, -1, y);
-        ycb = cb_index(g, y);
-        const su3<double> Ub = load_link<F64, double>(U, p ^ 1, mu, ycb);
-        v = load_spinor<F64, double>(other, j, ycb);
-        ph = x[mu] == 0 ? cx<double>{th.re[mu], -th.im[mu]} : cx<double>{1.0, 0.0};
-#pragma unroll
-        for (int s = 0; s < 4; ++s)
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-                acc.s[s][a] = acc.s[s][a] + ph * (cmul(Ub.m[0][a], v.s[s][0]) + cmul(Ub.m[1][a], v.s[s][1]) +
-                                                   cmul(Ub.m[2][a], v.s[s][2]));
+        const bool ph = (th.mask >> mu) & 1;
+        int y = cb_neighbour(g, x, mu, +1);
+        colour_hop<false>(acc, load_link<F64, double>(U, p, mu, cb), load_spinor<F64, double>(other, j, y),
+                          ph && x[mu] == g.L[mu] - 1, th.re[mu], th.im[mu]);
+        y = cb_neighbour(g, x, mu, -1);
+        colour_hop<true>(acc, load_link<F64, double>(U, p ^ 1, mu, y), load_spinor<F64, double>(other, j, y),
+                         ph && x[mu] == 0, th.re[mu], -th.im[mu]);
     }
+    const SpinorField<F64> self = in.h[p], s1 = a1.h[p], s2 = a2.h[p];
     const spinor<double> sv = load_spinor<F64, double>(self, j, cb);
     spinor<double> res;
 #pragma unroll
     for (int s = 0; s < 4; ++s)
 #pragma unroll
-        for (int a = 0; a < 3; ++a) res.s[s][a] = cH * acc.s[s][a] + c0 * sv.s[s][a];
-    if (a1.p) {
-        const spinor<double> av = load_spinor<F64, double>(a1, j, cb);
+        for (int a = 0; a < 3; ++a) res.s[s][a] = cd{fma(cH, acc.s[s][a].re, c0 * sv.s[s][a].re),
+                                                     fma(cH, acc.s[s][a].im, c0 * sv.s[s][a].im)};
+    if (s1.p) {
+        const spinor<double> av = load_spinor<F64, double>(s1, j, cb);
 #pragma unroll
         for (int s = 0; s < 4; ++s)
 #pragma unroll
-            for (int a = 0; a < 3; ++a) res.s[s][a] = res.s[s][a] + c1 * av.s[s][a];
+            for (int a = 0; a < 3; ++a) res.s[s][a] = cd{fma(c1, av.s[s][a].re, res.s[s][a].re),
+                                                         fma(c1, av.s[s][a].im, res.s[s][a].im)};
     }
-    if (a2.p) {
-        const spinor<double> av = load_spinor<F64, double>(a2, j, cb);
+    if (s2.p) {
+        const spinor<double> av = load_spinor<F64, double>(s2, j, cb);
 #pragma unroll
         for (int s = 0; s < 4; ++s)
 #pragma unroll
-            for (int a = 0; a < 3; ++a) res.s[s][a] = res.s[s][a] + c2 * av.s[s][a];
+            for (int a = 0; a < 3; ++a) res.s[s][a] = cd{fma(c2, av.s[s][a].re, res.s[s][a].re),
+                                                         fma(c2, av.s[s][a].im, res.s[s][a].im)};
     }
-    store_spinor<F64, double>(out, j, cb, res);
+    double2 *o = out.h[p].p + (long)j * 12 * out.h[p].stride + cb;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) o[k * out.h[p].stride] = make_double2(res.s[k / 3][k % 3].re, res.s[k / 3][k % 3].im);
 }
 
 // backflow combination: u = eta + z1; w = a u - c z2 (one parity, every RHS)
@@ -468,6 +685,7 @@ namespace {
 struct Full {
     SpinorField<F64> e, o;
     const SpinorField<F64> &half(int p) const { return p ? o : e; }
+    Halves halves() const { return Halves{{e, o}}; }
 };
 
 Full full_of(DevBuf &b, long stride, int nrhs)
@@ -484,14 +702,12 @@ static void laplace_stage(lqcd_lattice_s *lat, const LinkField<F64> &U, const Ph
                           const Full *a2 = nullptr, double c2 = 0.0)
 {
     // per output site and RHS: the spinor at 8 neighbours and itself (+ a1, a2), the output; 8 links per site
-    const double bytes = double(lat->vh) * (nrhs * 192.0 * (2.0 + (a1 ? 1.0 : 0.0) + (a2 ? 1.0 : 0.0)) + 8 * 144.0);
-    for (int p = 0; p < 2; ++p) {
-        ProfScope prof("fermion_flow_laplace", bytes, st);
-        laplace_kernel<<<unsigned(ntiles_of(lat->vh) * nrhs), kBlock, 0, st>>>(
-            lat->geom, p, U, th, in.half(p), in.half(p ^ 1), a1 ? a1->half(p) : SpinorField<F64>{},
-            a2 ? a2->half(p) : SpinorField<F64>{}, out.half(p), nrhs, cH, c0, c1, c2);
-        LQCD_CHECK_LAUNCH();
-    }
+    const double bytes = double(lat->V) * (nrhs * 192.0 * (2.0 + (a1 ? 1.0 : 0.0) + (a2 ? 1.0 : 0.0)) + 8 * 144.0);
+    ProfScope prof("fermion_flow_laplace", bytes, st);
+    laplace_kernel<<<dim3(unsigned(ntiles_of(lat->vh) * nrhs), 2), kBlock, 0, st>>>(
+        lat->geom, U, th, in.halves(), a1 ? a1->halves() : Halves{}, a2 ? a2->halves() : Halves{}, out.halves(), nrhs,
+        cH, c0, c1, c2);
+    LQCD_CHECK_LAUNCH();
 }
 
 void fermion_flow(lqcd_lattice_s *lat, GaugeSet &g, const lqcd_dirac_params &dp, double *psi_dev, int nrhs,
@@ -504,19 +720,19 @@ void fermion_flow(lqcd_lattice_s *lat, GaugeSet &g, const lqcd_dirac_params &dp,
     bchi.ensure(fb);
     bl1.ensure(fb);
     bl2.ensure(fb);
+    const FlowWork fw(S);
     const Full chi = full_of(bchi, S, nrhs), l1 = full_of(bl1, S, nrhs), l2 = full_of(bl2, S, nrhs);
-    Phases th;
-    hop_theta(dp, th.re, th.im);
+    const Phases th = phases_of(dp);
     const LinkField<F64> U{g.u64.as<const double2>(), nullptr, S};
     spinor_to_soa(lat, psi_dev, nrhs, chi.e, chi.o, st);
     for (int k = 0; k < nsteps; ++k) {
         laplace_stage(lat, U, th, chi, nullptr, l1, nrhs, 0.25 * eps, 1.0 - 2.0 * eps, 0.0, st);  // W0
-        flow_stage(lat, g.u64.as<double2>(), X.as<double2>(), 0, eps, st);
+        flow_stage(lat, g.u64.as<double2>(), X.as<double2>(), fw.s, 0, eps, st);
         laplace_stage(lat, U, th, l1, &chi, l2, nrhs, 8.0 / 9.0 * eps, -8.0 / 9.0 * (1.0 + 8.0 * eps), 17.0 / 9.0,
                       st);  // W1
-        flow_stage(lat, g.u64.as<double2>(), X.as<double2>(), 1, eps, st);
+        flow_stage(lat, g.u64.as<double2>(), X.as<double2>(), fw.s, 1, eps, st);
         laplace_stage(lat, U, th, l2, &l1, chi, nrhs, 0.75 * eps, -6.0 * eps, 1.0, st);  // W2
-        flow_stage(lat, g.u64.as<double2>(), X.as<double2>(), 2, eps, st);
+        flow_stage(lat, g.u64.as<double2>(), X.as<double2>(), fw.s, 2, eps, st);
     }
     spinor_from_soa(lat, psi_dev, nrhs, chi.e, chi.o, st);
     flow_finish(lat, g, st);
@@ -565,20 +781,12 @@ int hmc_trajectory(lqcd_lattice_s *lat, GaugeSet &g, double beta, double eps, in
     LQCD_CHECK_LAUNCH();
     const double H0 = kinetic_energy(lat, P.as<const double2>(), scratch.as<double>(), st) +
                       wilson_action(lat, g, beta, scratch.as<double>(), st);
-    const dim3 gf(unsigned((lat->vh + 63) / 64), 2, 4), gu(unsigned((lat->vh + 127) / 128), 2, 4);
-    const LinkField<F64> U{u64, nullptr, S};
-    const double fbytes = double(lat->V) * 4 * (8 * 144.0 + 144.0), lbytes = double(lat->V) * 4 * 3 * 144.0;
+    const FlowWork fw(S);
     for (int s = 0; s <= nsteps; ++s) {
-        const double h = (s == 0 || s == nsteps) ? 0.5 * eps : eps;  // P += h F(U), F = (beta / 6) Z
-        {
-            ProfScope prof("hmc_force", fbytes, st);
-            flow_force_kernel<<<gf, 64, 0, st>>>(lat->geom, U, P.as<double2>(), h * beta / 6.0, 1.0);
-            LQCD_CHECK_LAUNCH();
-        }
-        if (s == nsteps) break;
-        ProfScope prof("hmc_links", lbytes, st);  // U = exp(eps P) U
-        flow_update_kernel<<<gu, 128, 0, st>>>(lat->geom, u64, P.as<const double2>(), eps);
-        LQCD_CHECK_LAUNCH();
+        // P += h F(U), F = (beta / 6) Z, then U = exp(eps P) U (not after the last half step)
+        const double h = (s == 0 || s == nsteps) ? 0.5 * eps : eps;
+        force_step(lat, u64, P.as<double2>(), fw.s, h * beta / 6.0, 1.0, s == nsteps ? 0.0 : eps, "hmc_force",
+                   "hmc_links", st);
     }
     const double H1 = kinetic_energy(lat, P.as<const double2>(), scratch.as<double>(), st) +
                       wilson_action(lat, g, beta, scratch.as<double>(), st);
@@ -653,19 +861,19 @@ void fermion_backflow(lqcd_lattice_s *lat, GaugeSet &g, const lqcd_dirac_params 
     w1.ensure(ub);
     w2.ensure(ub);
     for (DevBuf *b : {&be, &bz1, &bz2, &bu, &bw}) b->ensure(fb);
+    const FlowWork fw(S);
     const Full eta = full_of(be, S, nrhs), z1 = full_of(bz1, S, nrhs), z2 = full_of(bz2, S, nrhs),
                u = full_of(bu, S, nrhs), w = full_of(bw, S, nrhs);
     const size_t nlink = ub / sizeof(double2);
     double2 *ckp = ck.as<double2>(), *segp = seg.as<double2>(), *W1 = w1.as<double2>(), *W2 = w2.as<double2>();
-    Phases th;
-    hop_theta(dp, th.re, th.im);
+    const Phases th = phases_of(dp);
     spinor_to_soa(lat, eta_dev, nrhs, eta.e, eta.o, st);
     // forward pass: checkpoints at the start of steps 0, m, 2m, ... (w1 is the running field)
     LQCD_CUDA(cudaMemcpyAsync(W1, g.u64.p, ub, cudaMemcpyDeviceToDevice, st));
     for (int k = 0; k < nsteps; ++k) {
         if (k % m == 0) LQCD_CUDA(cudaMemcpyAsync(ckp + (k / m) * nlink, W1, ub, cudaMemcpyDeviceToDevice, st));
         if (k + 1 < nsteps)  // the end field of the last step is not needed
-            for (int stage = 0; stage < 3; ++stage) flow_stage(lat, W1, X.as<double2>(), stage, eps, st);
+            for (int stage = 0; stage < 3; ++stage) flow_stage(lat, W1, X.as<double2>(), fw.s, stage, eps, st);
     }
     const double a = 0.25 * eps, b = 8.0 / 9.0 * eps, c = 2.0 / 9.0 * eps, d = 0.75 * eps;
     const unsigned gvec = unsigned(ntiles_of(lat->vh) * nrhs);
@@ -676,14 +884,14 @@ void fermion_backflow(lqcd_lattice_s *lat, GaugeSet &g, const lqcd_dirac_params 
         for (int k = k0 + 1; k < k1; ++k) {
             double2 *dst = segp + (k - k0) * nlink;
             LQCD_CUDA(cudaMemcpyAsync(dst, dst - nlink, ub, cudaMemcpyDeviceToDevice, st));
-            for (int stage = 0; stage < 3; ++stage) flow_stage(lat, dst, X.as<double2>(), stage, eps, st);
+            for (int stage = 0; stage < 3; ++stage) flow_stage(lat, dst, X.as<double2>(), fw.s, stage, eps, st);
         }
         for (int k = k1 - 1; k >= k0; --k) {
             double2 *W0 = segp + (k - k0) * nlink;
             LQCD_CUDA(cudaMemcpyAsync(W1, W0, ub, cudaMemcpyDeviceToDevice, st));
-            flow_stage(lat, W1, X.as<double2>(), 0, eps, st);
+            flow_stage(lat, W1, X.as<double2>(), fw.s, 0, eps, st);
             LQCD_CUDA(cudaMemcpyAsync(W2, W1, ub, cudaMemcpyDeviceToDevice, st));
-            flow_stage(lat, W2, X.as<double2>(), 1, eps, st);
+            flow_stage(lat, W2, X.as<double2>(), fw.s, 1, eps, st);
             const LinkField<F64> U0{W0, nullptr, S}, U1{W1, nullptr, S}, U2{W2, nullptr, S};
             laplace_stage(lat, U2, th, eta, nullptr, z2, nrhs, d, -8.0 * d, 0.0, st);  // z2 = d D2 eta
             laplace_stage(lat, U1, th, z2, nullptr, z1, nrhs, b, -8.0 * b, 0.0, st);   // z1 = b D1 z2
