@@ -3,6 +3,7 @@
 #pragma once
 #include <cstdlib>
 
+#include "hopd.cuh"
 #include "hopfast.cuh"
 #include "hopt.cuh"
 #include "lqcd_impl.h"
@@ -286,6 +287,28 @@ static FastHop<S> make_fast(const HopArgs<S, S, S> &a)
     return f;
 }
 
+// the small-lattice FP64 kernel (hopd.cuh); the norm's partials are per block of kSplitSites sites
+template <int MODE, bool NORM>
+static void hopd_go(const FastHop<F64> &f, CloverField<F64> clov2, double tau, bool dag, cudaStream_t st)
+{
+    const unsigned grid = unsigned(split_blocks(f.vh) * f.nrhs);
+    if (dag) hopd_kernel<MODE, true, NORM><<<grid, 128, 0, st>>>(f, clov2, tau);
+    else hopd_kernel<MODE, false, NORM><<<grid, 128, 0, st>>>(f, clov2, tau);
+}
+
+template <bool NORM>
+static void hopd_dispatch(const FastHop<F64> &f, CloverField<F64> clov2, double tau, int mode, bool dag,
+                          cudaStream_t st)
+{
+    switch (mode) {
+    case HOP_CLOV: hopd_go<HOP_CLOV, NORM>(f, clov2, tau, dag, st); break;
+    case SELF_CLOV: hopd_go<SELF_CLOV, NORM>(f, clov2, tau, dag, st); break;
+    case SELF_PLAIN: hopd_go<SELF_PLAIN, NORM>(f, clov2, tau, dag, st); break;
+    case CLOV_SUM: hopd_go<CLOV_SUM, NORM>(f, clov2, tau, dag, st); break;
+    default: hopd_go<RESID, NORM>(f, clov2, tau, dag, st); break;
+    }
+}
+
 template <class S, class L, class C, int MODE, bool DAG, bool NORM>
 static void hop_go(const HopArgs<S, L, C> &a, cudaStream_t st)
 {
@@ -324,6 +347,18 @@ void launch_hop(const HopArgs<S, L, C> &a, int mode, bool dag, bool norm, cudaSt
     const bool twinv = a.tau != 0.0 && (mode == HOP_CLOV || mode == CLOV_SUM);
     double shared = 8.0 * link_bytes<L>() + (mode == SELF_PLAIN ? 0.0 : (twinv ? 2.0 : 1.0) * clover_bytes<C>());
     const int pi = S::W == 2 ? 0 : (S::W == 4 ? 1 : 2);
+    if constexpr (std::is_same<S, F64>::value) {
+        if (split_hop(a.g.vh, a.nrhs)) {
+            {
+                ProfScope prof(kHopNames[pi][mode], double(a.g.vh) * (nact * per_rhs + (nact ? shared : 0.0)), st);
+                if (norm) hopd_dispatch<true>(make_fast(a), a.clov2, a.tau, mode, dag, st);
+                else hopd_dispatch<false>(make_fast(a), a.clov2, a.tau, mode, dag, st);
+                LQCD_CHECK_LAUNCH();
+            }
+            if (norm) launch_partial_finish(a.red, split_blocks(a.g.vh), a.nrhs, a.gate_st, a.gate, st);
+            return;
+        }
+    }
     // twisted mass runs on the generic kernel (hop_kernel) in every storage
     // format; the set-up and final modes have the fast kernel in FP64, without dagger
     const bool extra = std::is_same<S, F64>::value && !dag && (mode == SELF_PLAIN || mode == CLOV_SUM || mode == RESID);

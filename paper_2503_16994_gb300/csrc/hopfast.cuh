@@ -85,6 +85,16 @@ __device__ __forceinline__ void cmadc(R &ar, R &ai, R ur, R ui, R vr, R vi)
     ai = fma(-ui, vr, ai);
 }
 
+// (re, im) times the phase (pr, pi), as fmas, so that every FP64 kernel gives
+// the same bits
+template <typename R>
+__device__ __forceinline__ void phase_mul(R &re, R &im, R pr, R pi)
+{
+    const R xr = re, xi = im;
+    re = fma(-pi, xi, pr * xr);
+    im = fma(pi, xr, pr * xi);
+}
+
 // load the 24 reals of a spinor; for FP16 the values are returned unscaled
 // and the per-site scale separately (1 for FP32)
 template <class S, typename R>
@@ -496,11 +506,7 @@ __device__ __forceinline__ void dir_f(const FastHop<S> &a, const int (&jj)[NR], 
 #pragma unroll
             for (int s = 0; s < 2; ++s)
 #pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const R xr = gr[s][c], xi = gi[s][c];
-                    gr[s][c] = pr * xr - pi * xi;
-                    gi[s][c] = pr * xi + pi * xr;
-                }
+                for (int c = 0; c < 3; ++c) phase_mul(gr[s][c], gi[s][c], pr, pi);
         }
         accumulate_f<MU, SP, R>(acc[r], gr, gi);
     }

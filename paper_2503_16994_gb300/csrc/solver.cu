@@ -25,6 +25,7 @@
 #include <cmath>
 #include <cstdlib>
 
+#include "hopd.cuh"
 #include "lqcd_impl.h"
 
 namespace lqcd {
@@ -51,11 +52,13 @@ Workspace::~Workspace()
 
 // partial sums: the solver's reductions need nrhs * ntiles doubles followed
 // by the 4 nrhs ntiles FP32 partials of the tile hopping kernel (the room of
-// 2 nrhs ntiles doubles), the contraction T * ceil(V3/2 / 128) <= ntiles + T;
+// 2 nrhs ntiles doubles), on small batches one per block of the FP64 kernel
+// of hopd.cuh; the contraction T * ceil(V3/2 / 128) <= ntiles + T;
 // counters: max(nrhs, T)
 static size_t partial_count(const lqcd_lattice_s *lat, int nrhs)
 {
-    return std::max(3 * (size_t)nrhs * ntiles_of(lat->vh), (size_t)ntiles_of(lat->vh) + lat->dims[3]);
+    const size_t split = split_hop(lat->vh, nrhs) ? (size_t)nrhs * split_blocks(lat->vh) : 0;
+    return std::max({3 * (size_t)nrhs * ntiles_of(lat->vh), (size_t)ntiles_of(lat->vh) + lat->dims[3], split});
 }
 
 template <class W, class E>
