@@ -250,8 +250,9 @@ static HopShape hopf_tuned(FastHop<S> f, int mode, cudaStream_t st)
     return best;
 }
 
-template <class S>
-static FastHop<S> make_fast(const HopArgs<S, S, S> &a)
+// geometry, phases and coefficient of a launch, for any storage
+template <class S, class H>
+static FastHop<S> make_shape(const H &a)
 {
     FastHop<S> f{};
     for (int m = 0; m < 4; ++m) {
@@ -272,15 +273,24 @@ static FastHop<S> make_fast(const HopArgs<S, S, S> &a)
     f.oz = a.g.Lxh * a.g.L[1];
     f.ot = a.g.Lxh * a.g.L[1] * a.g.L[2];
     f.coef = a.coef;
+    f.tau = a.tau;
     f.gpb = 1;
     f.minb = 1;
     f.swz = 1;
+    return f;
+}
+
+template <class S>
+static FastHop<S> make_fast(const HopArgs<S, S, S> &a)
+{
+    FastHop<S> f = make_shape<S>(a);
     f.in = a.in;
     f.self = a.self;
     f.out = a.out;
     f.b = a.b;
     f.U = a.U;
     f.clov = a.clov;
+    f.site = a.site;
     f.gate_st = a.gate_st;
     f.gate = a.gate;
     f.red = a.red;
@@ -289,23 +299,22 @@ static FastHop<S> make_fast(const HopArgs<S, S, S> &a)
 
 // the small-lattice FP64 kernel (hopd.cuh); the norm's partials are per block of kSplitSites sites
 template <int MODE, bool NORM>
-static void hopd_go(const FastHop<F64> &f, CloverField<F64> clov2, double tau, bool dag, cudaStream_t st)
+static void hopd_go(const FastHop<F64> &f, CloverField<F64> clov2, bool dag, cudaStream_t st)
 {
     const unsigned grid = unsigned(split_blocks(f.vh) * f.nrhs);
-    if (dag) hopd_kernel<MODE, true, NORM><<<grid, 128, 0, st>>>(f, clov2, tau);
-    else hopd_kernel<MODE, false, NORM><<<grid, 128, 0, st>>>(f, clov2, tau);
+    if (dag) hopd_kernel<F64, MODE, true, NORM><<<grid, 128, 0, st>>>(f, clov2);
+    else hopd_kernel<F64, MODE, false, NORM><<<grid, 128, 0, st>>>(f, clov2);
 }
 
 template <bool NORM>
-static void hopd_dispatch(const FastHop<F64> &f, CloverField<F64> clov2, double tau, int mode, bool dag,
-                          cudaStream_t st)
+static void hopd_dispatch(const FastHop<F64> &f, CloverField<F64> clov2, int mode, bool dag, cudaStream_t st)
 {
     switch (mode) {
-    case HOP_CLOV: hopd_go<HOP_CLOV, NORM>(f, clov2, tau, dag, st); break;
-    case SELF_CLOV: hopd_go<SELF_CLOV, NORM>(f, clov2, tau, dag, st); break;
-    case SELF_PLAIN: hopd_go<SELF_PLAIN, NORM>(f, clov2, tau, dag, st); break;
-    case CLOV_SUM: hopd_go<CLOV_SUM, NORM>(f, clov2, tau, dag, st); break;
-    default: hopd_go<RESID, NORM>(f, clov2, tau, dag, st); break;
+    case HOP_CLOV: hopd_go<HOP_CLOV, NORM>(f, clov2, dag, st); break;
+    case SELF_CLOV: hopd_go<SELF_CLOV, NORM>(f, clov2, dag, st); break;
+    case SELF_PLAIN: hopd_go<SELF_PLAIN, NORM>(f, clov2, dag, st); break;
+    case CLOV_SUM: hopd_go<CLOV_SUM, NORM>(f, clov2, dag, st); break;
+    default: hopd_go<RESID, NORM>(f, clov2, dag, st); break;
     }
 }
 
@@ -351,8 +360,8 @@ void launch_hop(const HopArgs<S, L, C> &a, int mode, bool dag, bool norm, cudaSt
         if (split_hop(a.g.vh, a.nrhs)) {
             {
                 ProfScope prof(kHopNames[pi][mode], double(a.g.vh) * (nact * per_rhs + (nact ? shared : 0.0)), st);
-                if (norm) hopd_dispatch<true>(make_fast(a), a.clov2, a.tau, mode, dag, st);
-                else hopd_dispatch<false>(make_fast(a), a.clov2, a.tau, mode, dag, st);
+                if (norm) hopd_dispatch<true>(make_fast(a), a.clov2, mode, dag, st);
+                else hopd_dispatch<false>(make_fast(a), a.clov2, mode, dag, st);
                 LQCD_CHECK_LAUNCH();
             }
             if (norm) launch_partial_finish(a.red, split_blocks(a.g.vh), a.nrhs, a.gate_st, a.gate, st);

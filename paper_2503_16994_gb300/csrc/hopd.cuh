@@ -39,7 +39,8 @@ struct CloverRow {
     double2 o[5];
 };
 
-__device__ __forceinline__ void load_clover_row(const CloverField<F64> &f, int parity, int i, int blk, int r,
+template <class C>
+__device__ __forceinline__ void load_clover_row(const CloverField<C> &f, int parity, int i, int blk, int r,
                                                 CloverRow &A)
 {
     const double2 *b = f.p + ((long)parity * 36 + blk * 18) * f.stride + i;
@@ -67,10 +68,19 @@ __device__ __forceinline__ double2 clover_row(const CloverRow &A, const double2 
     return make_double2(re, im);
 }
 
-// tau: twisted mass of the site term (clov2: the C blocks of the twisted inverse, see HopArgs)
-template <int MODE, bool DAG, bool NORM>
-__global__ void __launch_bounds__(128) hopd_kernel(const FastHop<F64> a, const CloverField<F64> clov2, double tau)
+// clov2: the C blocks of the twisted inverse (see HopArgs).  S: F64, or A64
+// for both parities of host-layout fields in one launch (blockIdx.y).
+template <class S, int MODE, bool DAG, bool NORM>
+__global__ void __launch_bounds__(128) hopd_kernel(const FastHop<S> a, const CloverField<F64> clov2)
 {
+    constexpr bool HOST = std::is_same<S, A64>::value;
+    const int parity = HOST ? int(blockIdx.y) : a.parity;
+    const double tau = a.tau;
+    // the word of component 0 at a field's site, and the step to the next component
+    auto base = [&](const SpinorField<S> &f, int j, int cb, int odd) {
+        return HOST ? f.p + (long)spinor_site<S>(cb, odd) * 12 : f.p + (long)j * 12 * f.stride + cb;
+    };
+    auto step_of = [&](const SpinorField<S> &f) { return HOST ? 1L : f.stride; };
     __shared__ double2 part[8][12][kSplitSites];
     __shared__ double2 vec[12][kSplitSites];
     __shared__ double red[4];
@@ -84,14 +94,20 @@ __global__ void __launch_bounds__(128) hopd_kernel(const FastHop<F64> a, const C
     // the rows of the clover block are on their way while the hops run
     constexpr bool CLOV = MODE != SELF_PLAIN;
     constexpr bool INV = MODE == HOP_CLOV || MODE == CLOV_SUM;  // the block is an inverse: twisted by B and C
-    CloverRow A, A2;
+    CloverRow A, A2, As;
     if (CLOV && worker) {
-        load_clover_row(a.clov, a.parity, wi, comp / 6, comp % 6, A);
-        if (INV && tau != 0.0) load_clover_row(clov2, a.parity, wi, comp / 6, comp % 6, A2);
+        load_clover_row(a.clov, parity, wi, comp / 6, comp % 6, A);
+        if (INV && tau != 0.0) load_clover_row(clov2, parity, wi, comp / 6, comp % 6, A2);
+        if (MODE == CLOV_SUM && NORM) load_clover_row(a.site, parity, wi, comp / 6, comp % 6, As);
+    }
+    int wodd = 0;
+    if (HOST) {
+        const unsigned row = fdiv(unsigned(wi), a.dx), q1 = fdiv(row, a.dy), q2 = fdiv(q1, a.dz);
+        wodd = (parity + int(row - q1 * unsigned(a.L[1])) + int(q1 - q2 * unsigned(a.L[2])) + int(q2)) & 1;
     }
     double2 self = make_double2(0.0, 0.0);
     if (MODE != HOP_CLOV && worker) {
-        self = __ldg(a.self.p + ((long)j * 12 + comp) * a.self.stride + wi);
+        self = __ldg(base(a.self, j, wi, wodd) + comp * step_of(a.self));
         if (MODE == SELF_CLOV || MODE == RESID) vec[comp][wsite] = self;
     }
     {
@@ -104,7 +120,7 @@ __global__ void __launch_bounds__(128) hopd_kernel(const FastHop<F64> a, const C
         const unsigned q2 = fdiv(q1, a.dz);
         const int z = int(q1) - int(q2) * a.L[2];
         const int t = int(q2);
-        const int x = 2 * xh + ((a.parity + y + z + t) & 1);
+        const int odd = (parity + y + z + t) & 1, x = 2 * xh + odd;
         bool wrap;
         int n;
         if (mu == 0) {
@@ -118,8 +134,9 @@ __global__ void __launch_bounds__(128) hopd_kernel(const FastHop<F64> a, const C
             n = back ? i - step : i + step;
         }
         // the link W = U_mu(x), or U_mu(x - mu)^dag by the transposed planes and the sign of the imaginary parts
-        const double2 *up = a.U.p + (long)((back ? a.parity ^ 1 : a.parity) * 4 + mu) * 9 * a.U.stride + (back ? n : i);
-        const double2 *ip = a.in.p + (long)j * 12 * a.in.stride + n;
+        const double2 *up = a.U.p + (long)((back ? parity ^ 1 : parity) * 4 + mu) * 9 * a.U.stride + (back ? n : i);
+        const double2 *ip = base(a.in, j, n, mu == 0 ? 1 - odd : odd);
+        const long is = step_of(a.in);
         double2 w[3][3];
 #pragma unroll
         for (int r = 0; r < 3; ++r)
@@ -134,7 +151,7 @@ __global__ void __launch_bounds__(128) hopd_kernel(const FastHop<F64> a, const C
         double hr[3], hi[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const double2 u = __ldg(ip + (3 * s + c) * a.in.stride), d = __ldg(ip + (3 * (2 + o) + c) * a.in.stride);
+            const double2 u = __ldg(ip + (3 * s + c) * is), d = __ldg(ip + (3 * (2 + o) + c) * is);
             hr[c] = u.x + flip(im ? d.y : d.x, fneg != im);
             hi[c] = u.y + flip(im ? d.x : d.y, fneg);
         }
@@ -172,6 +189,7 @@ __global__ void __launch_bounds__(128) hopd_kernel(const FastHop<F64> a, const C
         __syncthreads();
     }
     double n2 = 0.0;
+    double2 out = make_double2(0.0, 0.0);
     if (wvalid) {
         const int blk = comp / 6, r = comp % 6;
         const double2 *v = &vec[6 * blk][wsite];
@@ -199,9 +217,25 @@ __global__ void __launch_bounds__(128) hopd_kernel(const FastHop<F64> a, const C
             const double2 b = __ldg(a.b.p + ((long)j * 12 + comp) * a.b.stride + wi);
             res = make_double2(b.x - res.x, b.y - res.y);
         } else {
-            a.out.p[((long)j * 12 + comp) * a.out.stride + wi] = res;
+            base(a.out, j, wi, wodd)[comp * step_of(a.out)] = res;
         }
         n2 = fma(res.x, res.x, res.y * res.y);
+        out = res;
+    }
+    if (MODE == CLOV_SUM && NORM) {  // |self + coef H in - A out|^2
+        __syncthreads();  // every row has read its input
+        const double2 v = worker ? vec[comp][wsite] : make_double2(0.0, 0.0);
+        __syncthreads();
+        if (worker) vec[comp][wsite] = out;
+        __syncthreads();
+        if (wvalid) {
+            const int blk = comp / 6;
+            const double ts = (blk == 0) != DAG ? tau : -tau;
+            double2 ao = clover_row(As, &vec[6 * blk][wsite], kSplitSites, comp % 6);
+            ao.x = fma(-ts, out.y, ao.x);
+            ao.y = fma(ts, out.x, ao.y);
+            n2 = fma(v.x - ao.x, v.x - ao.x, (v.y - ao.y) * (v.y - ao.y));
+        }
     }
     if (NORM) {
         n2 = warp_sum(n2);

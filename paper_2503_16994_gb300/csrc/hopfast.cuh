@@ -33,6 +33,11 @@ inline FastDiv make_fastdiv(unsigned d)
     return FastDiv{d, unsigned(m), l};
 }
 
+// FP64 spinors in the host layout (psi[site][24], lexicographic): no
+// right-hand side index, and sites are named by their lexicographic number.
+struct A64 { using word = double2; static constexpr int W = 2; };
+template <> struct spinor_planes<A64> { static constexpr int n = 12; };
+
 template <class S>
 struct FastHop {
     int L[4];
@@ -41,6 +46,7 @@ struct FastHop {
     int oy, oz, ot;              // cb offsets of one step in y, z, t
     double coef;
     double th_re[4], th_im[4];
+    double tau;                  // twisted mass of the site term (A64 and the small-batch kernel only)
     int gpb;                     // groups of NR right-hand sides per block
     int minb;                    // register cap: minimum resident blocks per SM (1, 4 or 6)
     int swz;                     // tiles per super-tile in the block order (1: tile-major)
@@ -48,6 +54,7 @@ struct FastHop {
     SpinorField<S> in, self, out, b;  // b: RESID only
     LinkField<S> U;
     CloverField<S> clov;
+    CloverField<S> site;  // CLOV_SUM with the norm: the site blocks A (FP64)
     const RhsState *gate_st;
     int gate;
     Reduce red;
@@ -65,6 +72,16 @@ inline long padded_tiles(const FastHop<S> &f)
 // ---------------------------------------------------------------------------
 template <typename R> struct real_of { using type = float; };
 template <> struct real_of<F64> { using type = double; };
+template <> struct real_of<A64> { using type = double; };
+
+// what a spinor field of storage S calls site cb of a parity; odd: (parity + y
+// + z + t) & 1 of that site, so that x = 2 xh + odd.  A hop in y, z or t keeps
+// it (parity and one coordinate change), a hop in x flips it.
+template <class S> __device__ __forceinline__ int spinor_site(int cb, int odd)
+{
+    if constexpr (std::is_same<S, A64>::value) return 2 * cb + odd;
+    else return cb;
+}
 
 // acc += u * v
 template <typename R>
@@ -102,7 +119,16 @@ __device__ __forceinline__ R load_raw(const SpinorField<S> &f, int j, int i, R v
 {
     constexpr int NP = spinor_planes<S>::n;
     const typename S::word *b = f.p + (long)j * NP * f.stride + i;
-    if constexpr (S::W == 2) {
+    if constexpr (std::is_same<S, A64>::value) {
+        b = f.p + (long)i * 12;
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+            const double2 w = __ldg(b + k);
+            v[2 * k] = w.x;
+            v[2 * k + 1] = w.y;
+        }
+        return R(1);
+    } else if constexpr (S::W == 2) {
 #pragma unroll
         for (int k = 0; k < NP; ++k) {
             double2 w = __ldg(b + k * f.stride);
@@ -144,7 +170,11 @@ __device__ __forceinline__ double store_raw(const SpinorField<S> &f, int j, int 
     constexpr int NP = spinor_planes<S>::n;
     typename S::word *b = f.p + (long)j * NP * f.stride + i;
     R n2 = R(0);
-    if constexpr (S::W == 2) {
+    if constexpr (std::is_same<S, A64>::value) {
+        b = f.p + (long)i * 12;
+#pragma unroll
+        for (int k = 0; k < NP; ++k) b[k] = make_double2(v[2 * k], v[2 * k + 1]);
+    } else if constexpr (S::W == 2) {
 #pragma unroll
         for (int k = 0; k < NP; ++k) {
             b[k * f.stride] = make_double2(v[2 * k], v[2 * k + 1]);
@@ -478,12 +508,25 @@ __device__ __forceinline__ void half_dir_rhs(const FastHop<S> &a, const float u[
     accumulate_sc<MU, SP>(acc, gr, gi, sc);
 }
 
-// one direction for all NR right-hand sides of this thread
-template <class S, int NR, int MU, int DIR, int SG, typename R>
-__device__ __forceinline__ void dir_f(const FastHop<S> &a, const int (&jj)[NR], unsigned on, int i, int y, bool wrap,
-                                      R (&acc)[NR][24])
+// one direction for all NR right-hand sides of this thread (odd: see spinor_site, of the output site)
+// SKIP: a hop whose inputs are zero in the whole warp adds nothing and is left out
+template <class S, int NR, int MU, int DIR, int SG, bool SKIP, typename R>
+__device__ __forceinline__ void dir_f(const FastHop<S> &a, const int (&jj)[NR], unsigned on, int i, int y, int odd,
+                                      bool wrap, R (&acc)[NR][24])
 {
     constexpr int SP = DIR > 0 ? -SG : SG;  // forward (1 - s g), backward (1 + s g)
+    if constexpr (SKIP) {
+        static_assert(S::W == 2, "FP64 only");
+        R v[24];
+        unsigned any = 0;  // on the words: FP64 comparisons would cost what the skip saves
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            load_raw<S, R>(a.in, jj[r], spinor_site<S>(y, MU == 0 ? 1 - odd : odd), v);
+#pragma unroll
+            for (int q = 0; q < 24; ++q) any |= unsigned(__double2loint(v[q])) | (unsigned(__double2hiint(v[q])) << 1);
+        }
+        if (!__any_sync(__activemask(), any != 0)) return;
+    }
     R u[18];
     load_link18<S, R>(a.U, DIR > 0 ? a.parity : (a.parity ^ 1), MU, DIR > 0 ? i : y, u);
     const bool ph = wrap && ((a.theta_mask >> MU) & 1);
@@ -497,7 +540,7 @@ __device__ __forceinline__ void dir_f(const FastHop<S> &a, const int (&jj)[NR], 
             continue;
         }
         R v[24];
-        const R sc = load_raw<S, R>(a.in, jj[r], y, v);
+        const R sc = load_raw<S, R>(a.in, jj[r], spinor_site<S>(y, MU == 0 ? 1 - odd : odd), v);
         R hr[2][3], hi[2][3], gr[2][3], gi[2][3];
         project_f<MU, SP, R>(v, hr, hi);
         link_mul<DIR < 0, R>(u, sc, hr, hi, gr, gi);
@@ -594,6 +637,7 @@ __device__ __forceinline__ void hopf_group(const FastHop<S> &a, int tile, int g)
     if (!on) return;
     const int i = tile * blockDim.x + threadIdx.x;
     const bool valid = i < a.vh;
+    int odd = 0;
     R acc[NR][24];
 #pragma unroll
     for (int r = 0; r < NR; ++r)
@@ -607,40 +651,43 @@ __device__ __forceinline__ void hopf_group(const FastHop<S> &a, int tile, int g)
         const unsigned q2 = fdiv(q1, a.dz);
         const int z = int(q1) - int(q2) * a.L[2];
         const int t = int(q2);
-        const int x = 2 * xh + ((a.parity + y + z + t) & 1);
+        odd = (a.parity + y + z + t) & 1;
+        const int x = 2 * xh + odd;
         const int rowbase = int(row) * a.Lxh;
         constexpr int SG = DAG ? -1 : 1;
+        // the set-up of a solve: b is a point source or a wall, zero almost everywhere
+        constexpr bool SKIP = MODE == SELF_PLAIN && S::W == 2;
         {
             const bool w = x == a.L[0] - 1;
-            dir_f<S, NR, 0, +1, SG, R>(a, jj, on, i, rowbase + ((w ? 0 : x + 1) >> 1), w, acc);
+            dir_f<S, NR, 0, +1, SG, SKIP, R>(a, jj, on, i, rowbase + ((w ? 0 : x + 1) >> 1), odd, w, acc);
         }
         {
             const bool w = x == 0;
-            dir_f<S, NR, 0, -1, SG, R>(a, jj, on, i, rowbase + ((w ? a.L[0] - 1 : x - 1) >> 1), w, acc);
+            dir_f<S, NR, 0, -1, SG, SKIP, R>(a, jj, on, i, rowbase + ((w ? a.L[0] - 1 : x - 1) >> 1), odd, w, acc);
         }
         {
             const bool w = y == a.L[1] - 1;
-            dir_f<S, NR, 1, +1, SG, R>(a, jj, on, i, i + (w ? -(a.L[1] - 1) * a.oy : a.oy), w, acc);
+            dir_f<S, NR, 1, +1, SG, SKIP, R>(a, jj, on, i, i + (w ? -(a.L[1] - 1) * a.oy : a.oy), odd, w, acc);
         }
         {
             const bool w = y == 0;
-            dir_f<S, NR, 1, -1, SG, R>(a, jj, on, i, i - (w ? -(a.L[1] - 1) * a.oy : a.oy), w, acc);
+            dir_f<S, NR, 1, -1, SG, SKIP, R>(a, jj, on, i, i - (w ? -(a.L[1] - 1) * a.oy : a.oy), odd, w, acc);
         }
         {
             const bool w = z == a.L[2] - 1;
-            dir_f<S, NR, 2, +1, SG, R>(a, jj, on, i, i + (w ? -(a.L[2] - 1) * a.oz : a.oz), w, acc);
+            dir_f<S, NR, 2, +1, SG, SKIP, R>(a, jj, on, i, i + (w ? -(a.L[2] - 1) * a.oz : a.oz), odd, w, acc);
         }
         {
             const bool w = z == 0;
-            dir_f<S, NR, 2, -1, SG, R>(a, jj, on, i, i - (w ? -(a.L[2] - 1) * a.oz : a.oz), w, acc);
+            dir_f<S, NR, 2, -1, SG, SKIP, R>(a, jj, on, i, i - (w ? -(a.L[2] - 1) * a.oz : a.oz), odd, w, acc);
         }
         {
             const bool w = t == a.L[3] - 1;
-            dir_f<S, NR, 3, +1, SG, R>(a, jj, on, i, i + (w ? -(a.L[3] - 1) * a.ot : a.ot), w, acc);
+            dir_f<S, NR, 3, +1, SG, SKIP, R>(a, jj, on, i, i + (w ? -(a.L[3] - 1) * a.ot : a.ot), odd, w, acc);
         }
         {
             const bool w = t == 0;
-            dir_f<S, NR, 3, -1, SG, R>(a, jj, on, i, i - (w ? -(a.L[3] - 1) * a.ot : a.ot), w, acc);
+            dir_f<S, NR, 3, -1, SG, SKIP, R>(a, jj, on, i, i - (w ? -(a.L[3] - 1) * a.ot : a.ot), odd, w, acc);
         }
     }
     // epilogue, one right-hand side at a time
@@ -654,7 +701,7 @@ __device__ __forceinline__ void hopf_group(const FastHop<S> &a, int tile, int g)
             if constexpr (MODE == SELF_PLAIN || MODE == CLOV_SUM) {
                 // self + coef H in, then (CLOV_SUM) times C
                 R sv[24];
-                const R sc = load_raw<S, R>(a.self, jj[r], i, sv);
+                const R sc = load_raw<S, R>(a.self, jj[r], spinor_site<S>(i, odd), sv);
                 if constexpr (S::W == 8) {
 #pragma unroll
                     for (int q = 0; q < 24; ++q) sv[q] *= sc;
@@ -671,6 +718,21 @@ __device__ __forceinline__ void hopf_group(const FastHop<S> &a, int tile, int g)
                         load_clov_block<S, R>(a.clov, a.parity, i, blk, A);
                         clov6(A, sv + 12 * blk, res + 12 * blk);
                     }
+                    if constexpr (NORM) {
+                        // |self + coef H in - A out|^2: the residual of the sites just solved
+                        R ao[12], t = R(0);
+#pragma unroll
+                        for (int blk = 0; blk < 2; ++blk) {
+                            load_clov_block<S, R>(a.site, a.parity, i, blk, A);
+                            clov6(A, res + 12 * blk, ao);
+#pragma unroll
+                            for (int q = 0; q < 12; ++q) {
+                                const R d = sv[12 * blk + q] - ao[q];
+                                t = fma(d, d, t);
+                            }
+                        }
+                        n2 = double(t);
+                    }
                 }
             } else if constexpr (MODE == HOP_CLOV) {
                 // out = coef * C (H in)
@@ -685,7 +747,7 @@ __device__ __forceinline__ void hopf_group(const FastHop<S> &a, int tile, int g)
             } else {
                 // out = C self + coef * H in
                 R sv[24];
-                const R sc = load_raw<S, R>(a.self, jj[r], i, sv);
+                const R sc = load_raw<S, R>(a.self, jj[r], spinor_site<S>(i, odd), sv);
                 if constexpr (S::W == 8) {
 #pragma unroll
                     for (int q = 0; q < 24; ++q) sv[q] *= sc;
@@ -695,6 +757,17 @@ __device__ __forceinline__ void hopf_group(const FastHop<S> &a, int tile, int g)
                 for (int blk = 0; blk < 2; ++blk) {
                     load_clov_block<S, R>(a.clov, a.parity, i, blk, A);
                     clov6(A, sv + 12 * blk, res + 12 * blk);
+                }
+                if constexpr (std::is_same<S, A64>::value) {
+                    if (a.tau != 0.0) {  // + i tau g5 self
+                        const R tau = DAG ? -a.tau : a.tau;
+#pragma unroll
+                        for (int q = 0; q < 12; ++q) {
+                            const R ts = q < 6 ? tau : -tau;
+                            res[2 * q] = fma(-ts, sv[2 * q + 1], res[2 * q]);
+                            res[2 * q + 1] = fma(ts, sv[2 * q], res[2 * q + 1]);
+                        }
+                    }
                 }
 #pragma unroll
                 for (int q = 0; q < 24; ++q) res[q] = fma(coef, acc[r][q], res[q]);
@@ -711,7 +784,8 @@ __device__ __forceinline__ void hopf_group(const FastHop<S> &a, int tile, int g)
                 }
                 n2 = double(t);
             } else {
-                n2 = store_raw<S, R>(a.out, jj[r], i, res);
+                const double s2 = store_raw<S, R>(a.out, jj[r], spinor_site<S>(i, odd), res);
+                if constexpr (MODE != CLOV_SUM) n2 = s2;
             }
         }
         if (NORM) {
@@ -748,6 +822,19 @@ __global__ void __launch_bounds__(128, MINB) hopf_kernel(const FastHop<S> a)
     const int g0 = gb * a.gpb;
     const int g1 = min(ngr, g0 + a.gpb);
     for (int g = g0; g < g1; ++g) hopf_group<S, NR, MODE, DAG, NORM>(a, tile, g);
+}
+
+// D psi (or D^dag psi) from and to the host layout, both parities in one
+// launch (blockIdx.y).  The FP64 pipe bounds it (1128 instructions a site), so
+// the uncoalesced reads of the host layout (120 16-byte accesses a site, each
+// a line of its own) stay hidden, and the two passes that converted the fields
+// fall away: 4.18 ms on 32^3 x 64 against 4.71, and 22 us on 4^4 (with
+// hopd_kernel) against 45.
+template <bool DAG>
+__global__ void __launch_bounds__(128) dirac_kernel(FastHop<A64> a)
+{
+    a.parity = blockIdx.y;
+    hopf_group<A64, 1, SELF_CLOV, DAG, false>(a, blockIdx.x, 0);
 }
 
 // ---------------------------------------------------------------------------

@@ -182,7 +182,7 @@ enum HopMode : int {
     HOP_CLOV = 0,   // out = coef * C (H in)
     SELF_CLOV = 1,  // out = C self + coef * H in
     SELF_PLAIN = 2, // out = self + coef * H in
-    CLOV_SUM = 3,   // out = C (self + coef * H in)
+    CLOV_SUM = 3,   // out = C (self + coef * H in), C an inverse; its norm is |self + coef * H in - A out|^2
     RESID = 4       // |b - (C self + coef * H in)|^2 only, nothing stored
 };
 
@@ -196,6 +196,7 @@ struct HopArgs {
     LinkField<L> U;
     CloverField<C> clov;   // clover blocks used by the epilogue (output parity taken from `parity`)
     CloverField<C> clov2;  // twisted mass: the C blocks of the inverse (clov then holds B), else unused
+    CloverField<C> site;   // CLOV_SUM with the norm: the site blocks A
     double tau;            // twisted mass 2 kappa mu of the site term (0: none); the dagger uses -tau
     double coef;
     double th_re[4], th_im[4];
@@ -322,6 +323,12 @@ __global__ void __launch_bounds__(128) hop_kernel(const HopArgs<S, L, C> a)
             } else {
                 res = clover_apply(blk, v);
             }
+            if constexpr (NORM) {
+                load_clover<C, R>(a.site, a.parity, i, blk);
+                spinor<R> ao = clover_apply(blk, res);
+                if (tau != R(0)) add_twist(ao, tau, res);
+                n2 = norm2_sp(axpy_sp(R(-1), ao, v));
+            }
         } else {  // SELF_CLOV, RESID
             clover_block<R> blk[2];
             load_clover<C, R>(a.clov, a.parity, i, blk);
@@ -335,7 +342,7 @@ __global__ void __launch_bounds__(128) hop_kernel(const HopArgs<S, L, C> a)
             n2 = norm2_sp(res);
         } else {
             double s2 = store_spinor<S, R>(a.out, j, i, res);
-            if (NORM) n2 = s2;
+            if (NORM && MODE != CLOV_SUM) n2 = s2;
         }
     }
     if (NORM) reduce_finish(a.red, j, tile, a.ntiles, n2);

@@ -251,6 +251,10 @@ void meson_contract(lqcd_lattice_s *lat, const double *prop_dev, int src_t, cons
 template <class S, class L, class C>
 void launch_hop(const HopArgs<S, L, C> &a, int mode, bool dag, bool norm, cudaStream_t st);
 
+// out = D in (or D^dag in) on fields in the host layout, FP64, device memory; a: geometry, links, phases, clover,
+// tau and coef = -kappa (dslash_f64.cu)
+void launch_dirac(const HopArgs<F64, F64, F64> &a, const double *in, double *out, bool dag, cudaStream_t st);
+
 // vector kernels (blas_*.cu)
 template <class W, class E>
 void launch_er_update(const VecArgs &v, SpinorField<W> p, SpinorField<W> w, SpinorField<W> r, SpinorField<E> e,

@@ -444,7 +444,10 @@ struct Solver {
         LQCD_CHECK_LAUNCH();
     }
 
-    // x_o = A_oo^-1 (b_o + k H_oe x_e); acc = |b - D x|^2 over both parities
+    // x_o = A_oo^-1 (b_o + k H_oe x_e); acc = |b - D x|^2 over both parities.
+    // On the odd sites the residual is (b_o + k H_oe x_e) - A_oo x_o, whose
+    // first part the solution has just been formed from, so the hop is not
+    // repeated for it.
     void finish()
     {
         HopArgs<F64, F64, F64> a = h64;
@@ -453,20 +456,16 @@ struct Solver {
         a.self = b_o;
         a.out = x_o;
         a.clov = ai64;
+        a.site = a64;
         a.coef = kappa;
-        launch_hop(a, CLOV_SUM, false, false, st);
+        a.red.op = RED_STORE;
+        launch_hop(a, CLOV_SUM, false, true, st);
         a.parity = 0;
         a.in = x_o;
         a.self = x_e;
         a.b = b_e;
         a.clov = a64;
         a.coef = -kappa;
-        a.red.op = RED_STORE;
-        launch_hop(a, RESID, false, true, st);
-        a.parity = 1;
-        a.in = x_e;
-        a.self = x_o;
-        a.b = b_o;
         a.red.op = RED_ADD;
         launch_hop(a, RESID, false, true, st);
     }
@@ -785,11 +784,7 @@ void dirac_apply_dev(lqcd_lattice_s *lat, GaugeSet &g, const lqcd_dirac_params &
                      bool dag, cudaStream_t st)
 {
     CloverSet &cl = clover_get(lat, g, dp, st);
-    Workspace &ws = workspace<F64, F64>(lat, 1, LQCD_PREC_FP64, st);
     const long Sd = lat->stride;
-    SpinorField<F64> ie = fld<F64>(ws.b_e, nullptr, Sd), io = fld<F64>(ws.b_o, nullptr, Sd);
-    SpinorField<F64> oe = fld<F64>(ws.x_e, nullptr, Sd), oo = fld<F64>(ws.x_o, nullptr, Sd);
-    spinor_to_soa(lat, in, 1, ie, io, st);
     HopArgs<F64, F64, F64> a{};
     a.g = lat->geom;
     a.nrhs = 1;
@@ -800,17 +795,7 @@ void dirac_apply_dev(lqcd_lattice_s *lat, GaugeSet &g, const lqcd_dirac_params &
     a.tau = cl.tau;
     a.coef = -dp.kappa;
     // (D psi)_p = A_p psi_p - kappa H_{p,1-p} psi_{1-p} on both parities
-    a.parity = 0;
-    a.in = io;
-    a.self = ie;
-    a.out = oe;
-    launch_hop(a, SELF_CLOV, dag, false, st);
-    a.parity = 1;
-    a.in = ie;
-    a.self = io;
-    a.out = oo;
-    launch_hop(a, SELF_CLOV, dag, false, st);
-    spinor_from_soa(lat, out, 1, oe, oo, st);
+    launch_dirac(a, in, out, dag, st);
 }
 
 template <class W, class E>

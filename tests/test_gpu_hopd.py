@@ -62,9 +62,11 @@ def test_both_kernels_store_the_same_bits(lq, theta):
         lq.lattice_destroy(lat)
 
 
-@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (6, 2, 6, 4)])
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (6, 2, 6, 4), (8, 8, 10, 14)])
 @pytest.mark.parametrize("mu", [0.0, 0.07])
-def test_solve_small(lq, dims, mu):
+def test_solve_reports_the_true_residual(lq, dims, mu):
+    """Three right-hand sides on either kernel (4480 sites are past the rule); the reported residual includes the
+    odd sites', which is formed with their solution."""
     U = inputs.gauge_field(dims, 0.3, seed=97)
     b = inputs.spinor_field(dims, seed=98, nrhs=3)
     lat = lq.lattice_create(dims)
