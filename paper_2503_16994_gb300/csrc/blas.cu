@@ -29,28 +29,35 @@ __device__ __forceinline__ double tile_partial(const Reduce &r, int j, int ntile
     }
 }
 
-// Sum of the per-tile partials of each gated-in RHS (one block of 512
-// threads per RHS, four independent accumulators per thread, fixed order:
-// deterministic) and its operation.
+// Sum of the per-tile partials of each gated-in RHS (one block per RHS, fixed
+// order: deterministic) and its operation.  One warp adds the threads' sums:
+// a shuffle tree in each of the 16 warps takes 80 FP64 instructions (16 cycles
+// each), twice the time of everything else at 4^4.
 constexpr int kFinishThreads = 512;
 template <bool QUAD>
 __global__ void __launch_bounds__(kFinishThreads) partial_finish_kernel(Reduce r, int ntiles, const RhsState *gate_st,
                                                                        int gate)
 {
-    __shared__ double sh[32];
+    __shared__ double sh[kFinishThreads];
+    pdl_begin();
     const int j = blockIdx.x;
     if (gate_st && gate_st[j].status != gate) return;
-    double t0 = 0.0, t1 = 0.0, t2 = 0.0, t3 = 0.0;
-    int k = threadIdx.x;
-    for (; k + 3 * kFinishThreads < ntiles; k += 4 * kFinishThreads) {
-        t0 += tile_partial<QUAD>(r, j, ntiles, k);
-        t1 += tile_partial<QUAD>(r, j, ntiles, k + kFinishThreads);
-        t2 += tile_partial<QUAD>(r, j, ntiles, k + 2 * kFinishThreads);
-        t3 += tile_partial<QUAD>(r, j, ntiles, k + 3 * kFinishThreads);
+    double t[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) t[q] = 0.0;
+    for (int k = threadIdx.x; k < ntiles; k += 8 * kFinishThreads) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (k + q * kFinishThreads < ntiles) t[q] += tile_partial<QUAD>(r, j, ntiles, k + q * kFinishThreads);
     }
-    for (; k < ntiles; k += kFinishThreads) t0 += tile_partial<QUAD>(r, j, ntiles, k);
-    double t = block_sum((t0 + t1) + (t2 + t3), sh);
-    if (threadIdx.x == 0) apply_op(r, j, t);
+    sh[threadIdx.x] = ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int k = 0; k < kFinishThreads / 32; ++k) s[k & 3] += sh[threadIdx.x + 32 * k];
+    const double sum = warp_sum((s[0] + s[1]) + (s[2] + s[3]));
+    if (threadIdx.x == 0) apply_op(r, j, sum);
 }
 
 void launch_partial_finish(const Reduce &r, int ntiles, int nrhs, const RhsState *gate_st, int gate, cudaStream_t st,
@@ -58,9 +65,9 @@ void launch_partial_finish(const Reduce &r, int ntiles, int nrhs, const RhsState
 {
     ProfScope prof("norm_finish", double(nrhs) * ntiles * (quad ? 16.0 : 8.0), st);
     if (quad)
-        partial_finish_kernel<true><<<unsigned(nrhs), kFinishThreads, 0, st>>>(r, ntiles, gate_st, gate);
+        launch_pdl(partial_finish_kernel<true>, dim3(unsigned(nrhs)), kFinishThreads, 0, st, r, ntiles, gate_st, gate);
     else
-        partial_finish_kernel<false><<<unsigned(nrhs), kFinishThreads, 0, st>>>(r, ntiles, gate_st, gate);
+        launch_pdl(partial_finish_kernel<false>, dim3(unsigned(nrhs)), kFinishThreads, 0, st, r, ntiles, gate_st, gate);
     LQCD_CHECK_LAUNCH();
 }
 
@@ -74,7 +81,10 @@ void launch_er_update(const VecArgs &v, SpinorField<W> p, SpinorField<W> w, Spin
 {
     ProfScope prof(prec_name<W>() == std::string("f64") ? "cg_er_update_f64" : (prec_name<W>() == std::string("f32") ? "cg_er_update_f32" : "cg_er_update_f16"),
                    double(v.vh) * nact(v) * (4.0 * spinor_bytes<W>() + 2.0 * spinor_bytes<E>()), st);
-    cg_er_update<W, E><<<grid_of(v), kBlock, 0, st>>>(v, p, w, r, e);
+    if constexpr (std::is_same<W, F64>::value)
+        launch_pdl(cg_er_update<W, E>, dim3(grid_of(v)), kBlock, 0, st, v, p, w, r, e);
+    else
+        cg_er_update<W, E><<<grid_of(v), kBlock, 0, st>>>(v, p, w, r, e);
     LQCD_CHECK_LAUNCH();
 }
 
@@ -82,7 +92,10 @@ template <class W>
 void launch_p_update(const VecArgs &v, const RhsState *s, SpinorField<W> z, SpinorField<W> p, cudaStream_t st)
 {
     ProfScope prof("cg_p_update", double(v.vh) * nact(v) * 3.0 * spinor_bytes<W>(), st);
-    cg_p_update<W><<<grid_of(v), kBlock, 0, st>>>(v, s, z, p);
+    if constexpr (std::is_same<W, F64>::value)
+        launch_pdl(cg_p_update<W>, dim3(grid_of(v)), kBlock, 0, st, v, s, z, p);
+    else
+        cg_p_update<W><<<grid_of(v), kBlock, 0, st>>>(v, s, z, p);
     LQCD_CHECK_LAUNCH();
 }
 

@@ -302,8 +302,8 @@ template <int MODE, bool NORM>
 static void hopd_go(const FastHop<F64> &f, CloverField<F64> clov2, bool dag, cudaStream_t st)
 {
     const unsigned grid = unsigned(split_blocks(f.vh) * f.nrhs);
-    if (dag) hopd_kernel<F64, MODE, true, NORM><<<grid, 128, 0, st>>>(f, clov2);
-    else hopd_kernel<F64, MODE, false, NORM><<<grid, 128, 0, st>>>(f, clov2);
+    if (dag) launch_pdl(hopd_kernel<F64, MODE, true, NORM>, dim3(grid), 128, 0, st, f, clov2);
+    else launch_pdl(hopd_kernel<F64, MODE, false, NORM>, dim3(grid), 128, 0, st, f, clov2);
 }
 
 template <bool NORM>

@@ -73,6 +73,7 @@ __device__ __forceinline__ double2 clover_row(const CloverRow &A, const double2 
 template <class S, int MODE, bool DAG, bool NORM>
 __global__ void __launch_bounds__(128) hopd_kernel(const FastHop<S> a, const CloverField<F64> clov2)
 {
+    pdl_begin();
     constexpr bool HOST = std::is_same<S, A64>::value;
     const int parity = HOST ? int(blockIdx.y) : a.parity;
     const double tau = a.tau;
@@ -107,7 +108,7 @@ __global__ void __launch_bounds__(128) hopd_kernel(const FastHop<S> a, const Clo
     }
     double2 self = make_double2(0.0, 0.0);
     if (MODE != HOP_CLOV && worker) {
-        self = __ldg(base(a.self, j, wi, wodd) + comp * step_of(a.self));
+        self = *(base(a.self, j, wi, wodd) + comp * step_of(a.self));
         if (MODE == SELF_CLOV || MODE == RESID) vec[comp][wsite] = self;
     }
     {
@@ -151,7 +152,7 @@ __global__ void __launch_bounds__(128) hopd_kernel(const FastHop<S> a, const Clo
         double hr[3], hi[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const double2 u = __ldg(ip + (3 * s + c) * is), d = __ldg(ip + (3 * (2 + o) + c) * is);
+            const double2 u = *(ip + (3 * s + c) * is), d = *(ip + (3 * (2 + o) + c) * is);
             hr[c] = u.x + flip(im ? d.y : d.x, fneg != im);
             hi[c] = u.y + flip(im ? d.x : d.y, fneg);
         }
@@ -214,7 +215,7 @@ __global__ void __launch_bounds__(128) hopd_kernel(const FastHop<S> a, const Clo
             res = make_double2(fma(coef, H.x, res.x), fma(coef, H.y, res.y));
         }
         if (MODE == RESID) {
-            const double2 b = __ldg(a.b.p + ((long)j * 12 + comp) * a.b.stride + wi);
+            const double2 b = a.b.p[((long)j * 12 + comp) * a.b.stride + wi];
             res = make_double2(b.x - res.x, b.y - res.y);
         } else {
             base(a.out, j, wi, wodd)[comp * step_of(a.out)] = res;

@@ -30,6 +30,7 @@ struct RhsState {
     int updates;
     int maxiter;
     int resume;      // status after an FP64 residual that did not finish: ST_ACTIVE or ST_RESUME
+    float alpha_f, beta_f;  // alpha, beta in FP32 (the FP16/FP32 vector kernels; converted once)
 };
 
 // What the last block does with a finished per-RHS sum.
@@ -57,9 +58,13 @@ __device__ __forceinline__ void apply_op(const Reduce &r, int j, double sum)
     switch (r.op) {
     case RED_STORE: s.acc = sum; break;
     case RED_ADD: s.acc += sum; break;
-    case RED_ALPHA: s.alpha = sum > 0.0 ? s.gamma / sum : 0.0; break;
+    case RED_ALPHA:
+        s.alpha = sum > 0.0 ? s.gamma / sum : 0.0;
+        s.alpha_f = float(s.alpha);
+        break;
     case RED_BETA:
         s.beta = s.gamma > 0.0 ? sum / s.gamma : 0.0;
+        s.beta_f = float(s.beta);
         s.gamma = sum;
         break;
     case RED_RUPDATE:
@@ -89,14 +94,31 @@ __device__ __forceinline__ void apply_op(const Reduce &r, int j, double sum)
     }
 }
 
+// Sum of v over a block of at most 128 threads (result valid in warp 0).  The
+// values meet in shared memory and one warp adds them, four to a lane: 8 FP64
+// instructions of a warp instead of the 25 of a shuffle tree in every warp
+// (block_sum).  An FP64 instruction takes this GPU's SM 16 cycles, so the
+// tree of every block is 0.2 us of its SM.
+__device__ __forceinline__ double block_sum4(double v, double *sh)
+{
+    __syncthreads();
+    sh[threadIdx.x] = v;
+    __syncthreads();
+    if (threadIdx.x >= 32) return 0.0;
+    double t[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) t[k] = threadIdx.x + 32 * k < blockDim.x ? sh[threadIdx.x + 32 * k] : 0.0;
+    return warp_sum((t[0] + t[1]) + (t[2] + t[3]));
+}
+
 // Block-wide sum of v, written as this block's partial; the last block of
 // RHS j to arrive sums all partials in a fixed order (deterministic) and
-// applies the operation.  Must be called by every thread of the block.
+// applies the operation.  Must be called by every thread of the block (128).
 __device__ __forceinline__ void reduce_finish(const Reduce &r, int j, int tile, int ntiles, double v)
 {
-    __shared__ double sh[32];
+    __shared__ double sh[128];
     __shared__ int last;
-    double s = block_sum(v, sh);
+    double s = block_sum4(v, sh);
     if (threadIdx.x == 0) {
         r.partial[(long)j * ntiles + tile] = s;
         __threadfence();
@@ -108,7 +130,7 @@ __device__ __forceinline__ void reduce_finish(const Reduce &r, int j, int tile, 
         __threadfence();
         double t = 0.0;
         for (int k = threadIdx.x; k < ntiles; k += blockDim.x) t += __ldcg(r.partial + (long)j * ntiles + k);
-        t = block_sum(t, sh);
+        t = block_sum4(t, sh);
         if (threadIdx.x == 0) {
             r.counter[j] = 0;
             apply_op(r, j, t);
@@ -359,24 +381,58 @@ struct VecArgs {
     int nactive = -1;  // launch accounting only: right-hand sides expected to pass the gate (-1: all)
 };
 
+// an FP64 spinor by plain loads (a field that the same launch, or one in flight, also writes)
+__device__ __forceinline__ spinor<double> load_spinor_f64_rw(const SpinorField<F64> &f, int j, int i)
+{
+    spinor<double> a;
+    double *v = reinterpret_cast<double *>(&a);
+    const double2 *b = f.p + (long)j * 12 * f.stride + i;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        const double2 w = b[k * f.stride];
+        v[2 * k] = w.x;
+        v[2 * k + 1] = w.y;
+    }
+    return a;
+}
+
+// a vector of the CG update kernels: FP64 ones are launched while the kernel
+// before them still runs (launch_pdl), so they are read by plain loads
+template <class S, typename R>
+__device__ __forceinline__ spinor<R> load_vec(const SpinorField<S> &f, int j, int i)
+{
+    if constexpr (std::is_same<S, F64>::value && std::is_same<R, double>::value) return load_spinor_f64_rw(f, j, i);
+    else return load_spinor<S, R>(f, j, i);
+}
+
 // e += alpha p ; r -= alpha w ; |r|^2 -> RED_RUPDATE
+template <typename R> __device__ __forceinline__ R alpha_of(const RhsState &s)
+{
+    if constexpr (std::is_same<R, float>::value) return s.alpha_f;
+    else return s.alpha;
+}
+template <typename R> __device__ __forceinline__ R beta_of(const RhsState &s)
+{
+    if constexpr (std::is_same<R, float>::value) return s.beta_f;
+    else return s.beta;
+}
+
 template <class W, class E>
 __global__ void __launch_bounds__(128) cg_er_update(VecArgs v, SpinorField<W> p, SpinorField<W> w, SpinorField<W> r,
                                                     SpinorField<E> e)
 {
+    pdl_begin();
     const int j = blockIdx.x % v.nrhs, tile = blockIdx.x / v.nrhs;
     if (v.gate_st && v.gate_st[j].status != v.gate) return;
     const int i = tile * blockDim.x + threadIdx.x;
     double n2 = 0.0;
     if (i < v.vh) {
-        const double al = v.red.st[j].alpha;
         using R = typename std::conditional<std::is_same<E, F64>::value, double, float>::type;
-        spinor<R> pv = load_spinor<W, R>(p, j, i);
-        spinor<R> ev = load_spinor<E, R>(e, j, i);
-        store_spinor<E, R>(e, j, i, axpy_sp(R(al), pv, ev));
-        spinor<R> wv = load_spinor<W, R>(w, j, i);
-        spinor<R> rv = load_spinor<W, R>(r, j, i);
-        n2 = store_spinor<W, R>(r, j, i, axpy_sp(R(-al), wv, rv));
+        const R al = alpha_of<R>(v.red.st[j]);
+        const spinor<R> pv = load_vec<W, R>(p, j, i), ev = load_vec<E, R>(e, j, i);
+        const spinor<R> wv = load_vec<W, R>(w, j, i), rv = load_vec<W, R>(r, j, i);
+        store_spinor<E, R>(e, j, i, axpy_sp(al, pv, ev));
+        n2 = store_spinor<W, R>(r, j, i, axpy_sp(-al, wv, rv));
     }
     reduce_finish(v.red, j, tile, v.ntiles, n2);
 }
@@ -385,13 +441,13 @@ __global__ void __launch_bounds__(128) cg_er_update(VecArgs v, SpinorField<W> p,
 template <class W>
 __global__ void __launch_bounds__(128) cg_p_update(VecArgs v, const RhsState *st, SpinorField<W> z, SpinorField<W> p)
 {
+    pdl_begin();
     const int j = blockIdx.x % v.nrhs, tile = blockIdx.x / v.nrhs;
     if (v.gate_st && v.gate_st[j].status != v.gate) return;
     const int i = tile * blockDim.x + threadIdx.x;
     if (i >= v.vh) return;
     using R = typename std::conditional<std::is_same<W, F64>::value, double, float>::type;
-    const double be = st[j].beta;
-    store_spinor<W, R>(p, j, i, axpy_sp(R(be), load_spinor<W, R>(p, j, i), load_spinor<W, R>(z, j, i)));
+    store_spinor<W, R>(p, j, i, axpy_sp(beta_of<R>(st[j]), load_vec<W, R>(p, j, i), load_vec<W, R>(z, j, i)));
 }
 
 // x += scale e ; e = 0   (FP64 x)
@@ -408,21 +464,6 @@ __global__ void __launch_bounds__(128) cg_x_update(VecArgs v, const RhsState *st
     spinor<double> z;
     zero(z);
     store_spinor<E, double>(e, j, i, z);
-}
-
-// an FP64 spinor through the coherent path (a field the same launch also writes)
-__device__ __forceinline__ spinor<double> load_spinor_f64_rw(const SpinorField<F64> &f, int j, int i)
-{
-    spinor<double> a;
-    double *v = reinterpret_cast<double *>(&a);
-    const double2 *b = f.p + (long)j * 12 * f.stride + i;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        const double2 w = b[k * f.stride];
-        v[2 * k] = w.x;
-        v[2 * k + 1] = w.y;
-    }
-    return a;
 }
 
 // rhat = src - c w (FP64 arithmetic): the FP64 update has src = bhat, w =

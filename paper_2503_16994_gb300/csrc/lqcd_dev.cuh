@@ -24,6 +24,18 @@
 
 namespace lqcd {
 
+// First statement of a kernel launched by launch_pdl: waits until the kernel
+// before it on the stream has ended and its writes are visible, then lets the
+// next one's blocks be scheduled as soon as all of this one's are.  Nothing in
+// device memory is touched before it, and what the kernel before may have
+// written (spinors, scales, states) is read by plain loads: the read-only path
+// (__ldg) is for data no kernel in flight writes, links and clover blocks.
+__device__ __forceinline__ void pdl_begin()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---------------------------------------------------------------------------
 // complex numbers
 // ---------------------------------------------------------------------------

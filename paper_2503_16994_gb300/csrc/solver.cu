@@ -146,6 +146,7 @@ __global__ void init_state_kernel(RhsState *s, int nrhs, double tol2, double del
     q.maxiter = maxiter;
     q.status = q.bnorm2 > 0.0 ? ST_UPDATE : ST_DONE;
     q.gamma = q.alpha = q.beta = 0.0;
+    q.alpha_f = q.beta_f = 0.f;
     q.rr = q.rr_ref = q.anchor2 = 0.0;
     q.iter = 0;
     q.updates = -1;  // the first FP64 residual (of the zero start) is not an update
