@@ -15,11 +15,27 @@ static void hopf_go(const FastHop<S> &f, cudaStream_t st)
 {
     const int ngr = (f.nrhs + NR - 1) / NR;
     const unsigned grid = unsigned(padded_tiles(f) * ((ngr + f.gpb - 1) / f.gpb));
-    // minimum resident blocks per SM (register cap) as chosen by the autotuner
-    if (NR == 1 && f.minb >= 6)
-        hopf_kernel<S, NR, MODE, DAG, NORM, 6><<<grid, kBlock, 0, st>>>(f);
-    else
-        hopf_kernel<S, NR, MODE, DAG, NORM, 1><<<grid, kBlock, 0, st>>>(f);
+    // minimum resident blocks per SM (register cap) as chosen by the autotuner (FP64: none)
+    if constexpr (NR == 1 && !std::is_same<S, F64>::value) {
+        if (f.minb >= 6) {
+            hopf_kernel<S, NR, MODE, DAG, NORM, 6><<<grid, kBlock, 0, st>>>(f);
+            return;
+        }
+    }
+    hopf_kernel<S, NR, MODE, DAG, NORM, 1><<<grid, kBlock, 0, st>>>(f);
+}
+
+template <class S, int NR, int MODE>
+static void hopf_mode(const FastHop<S> &f, bool dag, bool norm, cudaStream_t st)
+{
+    if (dag) norm ? hopf_go<S, NR, MODE, true, true>(f, st) : hopf_go<S, NR, MODE, true, false>(f, st);
+    else norm ? hopf_go<S, NR, MODE, false, true>(f, st) : hopf_go<S, NR, MODE, false, false>(f, st);
+}
+
+template <class S, int NR, int MODE>
+static void hopf_nodag(const FastHop<S> &f, bool norm, cudaStream_t st)
+{
+    norm ? hopf_go<S, NR, MODE, false, true>(f, st) : hopf_go<S, NR, MODE, false, false>(f, st);
 }
 
 template <class S, int NR>
@@ -27,26 +43,26 @@ static void hopf_dispatch(const FastHop<S> &f, int mode, bool dag, bool norm, cu
 {
     if constexpr (std::is_same<S, F64>::value) {
         // the FP64 set-up and final modes of the solver (no dagger)
-        if (mode == SELF_PLAIN) {
-            norm ? hopf_go<S, NR, SELF_PLAIN, false, true>(f, st) : hopf_go<S, NR, SELF_PLAIN, false, false>(f, st);
+        switch (mode) {
+        case SELF_PLAIN: hopf_nodag<S, NR, SELF_PLAIN>(f, norm, st); return;
+        case CLOV_SUM: hopf_nodag<S, NR, CLOV_SUM>(f, norm, st); return;
+        case RESID: hopf_nodag<S, NR, RESID>(f, norm, st); return;
+        case CLOV_SUM + TWIST: hopf_nodag<S, NR, CLOV_SUM + TWIST>(f, norm, st); return;
+        case RESID + TWIST: hopf_nodag<S, NR, RESID + TWIST>(f, norm, st); return;
+        }
+    }
+    if constexpr (NR == 1) {  // twisted mass: one right-hand side per thread, or the paired kernel
+        if (mode == HOP_CLOV + TWIST) {
+            hopf_mode<S, NR, HOP_CLOV + TWIST>(f, dag, norm, st);
             return;
         }
-        if (mode == CLOV_SUM) {
-            norm ? hopf_go<S, NR, CLOV_SUM, false, true>(f, st) : hopf_go<S, NR, CLOV_SUM, false, false>(f, st);
-            return;
-        }
-        if (mode == RESID) {
-            norm ? hopf_go<S, NR, RESID, false, true>(f, st) : hopf_go<S, NR, RESID, false, false>(f, st);
+        if (mode == SELF_CLOV + TWIST) {
+            hopf_mode<S, NR, SELF_CLOV + TWIST>(f, dag, norm, st);
             return;
         }
     }
-    if (mode == HOP_CLOV) {
-        if (dag) norm ? hopf_go<S, NR, HOP_CLOV, true, true>(f, st) : hopf_go<S, NR, HOP_CLOV, true, false>(f, st);
-        else norm ? hopf_go<S, NR, HOP_CLOV, false, true>(f, st) : hopf_go<S, NR, HOP_CLOV, false, false>(f, st);
-    } else {
-        if (dag) norm ? hopf_go<S, NR, SELF_CLOV, true, true>(f, st) : hopf_go<S, NR, SELF_CLOV, true, false>(f, st);
-        else norm ? hopf_go<S, NR, SELF_CLOV, false, true>(f, st) : hopf_go<S, NR, SELF_CLOV, false, false>(f, st);
-    }
+    if (mode == HOP_CLOV) hopf_mode<S, NR, HOP_CLOV>(f, dag, norm, st);
+    else hopf_mode<S, NR, SELF_CLOV>(f, dag, norm, st);
 }
 
 // paired kernels: instantiated in hopp_f16.cu / hopp_f32.cu (own translation
@@ -133,9 +149,12 @@ struct HopShape {
     int nr, gpb, minb, swz;
 };
 
+// Twisted mass (mode + TWIST) has the shapes nr = 0 and 1; its choices are
+// made per process (neither imported nor reported).
 template <class S>
 static HopShape hopf_tuned(FastHop<S> f, int mode, cudaStream_t st)
 {
+    const bool tw = mode >= TWIST;
     static std::mutex mu;
     static std::map<std::tuple<int, int, int, int>, HopShape> table;
     const char *env_nr = std::getenv("LQCD_HOP_NR");
@@ -145,6 +164,7 @@ static HopShape hopf_tuned(FastHop<S> f, int mode, cudaStream_t st)
         const bool staged = std::is_same<S, F16>::value && (nr == 12 || nr == 13 || is_tile_shape(nr));
         if (std::is_same<S, F64>::value || (!staged && nr != -2 && nr != -4 && nr != -8 && (nr < 0 || nr > 3)))
             nr = 1;
+        if (tw && nr != 0) nr = 1;
         if (is_tile_shape(nr) && !env_gpb) gpb = std::min(kTileMaxPairs, (f.nrhs + 1) / 2);
         const char *env_mb = std::getenv("LQCD_HOP_MINB");
         const char *env_sw = std::getenv("LQCD_HOP_SWZ");
@@ -159,7 +179,7 @@ static HopShape hopf_tuned(FastHop<S> f, int mode, cudaStream_t st)
     {
         // a shape imported from an earlier process (lqcd_tune_import) is used as is
         int sh[4];
-        if (tune_imported(prec_name<S>(), mode, f.vh, f.nrhs, sh)) {
+        if (!tw && tune_imported(prec_name<S>(), mode, f.vh, f.nrhs, sh)) {
             const HopShape h{sh[0], sh[1], sh[2], sh[3]};
             std::lock_guard<std::mutex> lk(mu);
             if (table.emplace(key, h).second)
@@ -177,7 +197,7 @@ static HopShape hopf_tuned(FastHop<S> f, int mode, cudaStream_t st)
         if (it != table.end()) return it->second;
     }
     std::vector<HopShape> cand;
-    const int maxnr = std::is_same<S, F64>::value ? 1 : 3;
+    const int maxnr = std::is_same<S, F64>::value || tw ? 1 : 3;
     for (int nr = (std::is_same<S, F64>::value || f.nrhs < 2) ? 1 : 0; nr <= maxnr && nr <= f.nrhs; ++nr) {
         const int per = nr == 0 ? 2 : nr;
         const int ngr = (f.nrhs + per - 1) / per;
@@ -199,7 +219,7 @@ static HopShape hopf_tuned(FastHop<S> f, int mode, cudaStream_t st)
                 }
             }
     }
-    if (std::is_same<S, F16>::value && f.nrhs >= 2) {
+    if (std::is_same<S, F16>::value && f.nrhs >= 2 && !tw) {
         const int ngr = (f.nrhs + 1) / 2;
         for (int gpb : {1, 2, 3, 6})
             if (gpb <= ngr && (gpb == 1 || ngr % gpb == 0)) {
@@ -208,7 +228,7 @@ static HopShape hopf_tuned(FastHop<S> f, int mode, cudaStream_t st)
                 cand.push_back(HopShape{13, gpb, 3, 1});
             }
     }
-    if (!std::is_same<S, F64>::value)
+    if (!std::is_same<S, F64>::value && !tw)
         for (int pf : {2, 4, 8})
             for (int gpb : {1, 2, 3})
                 if (gpb <= f.nrhs && (gpb == 1 || f.nrhs % gpb == 0)) cand.push_back(HopShape{-pf, gpb, 1, 1});
@@ -246,7 +266,7 @@ static HopShape hopf_tuned(FastHop<S> f, int mode, cudaStream_t st)
     LQCD_CHECK_LAUNCH();
     std::lock_guard<std::mutex> lk(mu);
     table[key] = best;
-    tune_record(prec_name<S>(), mode, f.vh, f.nrhs, best.nr, best.gpb, best.minb, best.swz, best_ms);
+    if (!tw) tune_record(prec_name<S>(), mode, f.vh, f.nrhs, best.nr, best.gpb, best.minb, best.swz, best_ms);
     return best;
 }
 
@@ -290,6 +310,7 @@ static FastHop<S> make_fast(const HopArgs<S, S, S> &a)
     f.b = a.b;
     f.U = a.U;
     f.clov = a.clov;
+    f.clov2 = a.clov2;
     f.site = a.site;
     f.gate_st = a.gate_st;
     f.gate = a.gate;
@@ -316,27 +337,6 @@ static void hopd_dispatch(const FastHop<F64> &f, CloverField<F64> clov2, int mod
     case CLOV_SUM: hopd_go<CLOV_SUM, NORM>(f, clov2, dag, st); break;
     default: hopd_go<RESID, NORM>(f, clov2, dag, st); break;
     }
-}
-
-template <class S, class L, class C, int MODE, bool DAG, bool NORM>
-static void hop_go(const HopArgs<S, L, C> &a, cudaStream_t st)
-{
-    using R = typename std::conditional<std::is_same<S, F64>::value, double, float>::type;
-    hop_kernel<S, L, C, R, MODE, DAG, NORM><<<unsigned(a.ntiles * a.nrhs), kBlock, 0, st>>>(a);
-}
-
-template <class S, class L, class C, int MODE>
-static bool hop_mode(const HopArgs<S, L, C> &a, int mode, bool dag, bool norm, cudaStream_t st)
-{
-    if (mode != MODE) return false;
-    if (dag) {
-        if (norm) hop_go<S, L, C, MODE, true, true>(a, st);
-        else hop_go<S, L, C, MODE, true, false>(a, st);
-    } else {
-        if (norm) hop_go<S, L, C, MODE, false, true>(a, st);
-        else hop_go<S, L, C, MODE, false, false>(a, st);
-    }
-    return true;
 }
 
 static const char *const kHopNames[3][5] = {
@@ -368,38 +368,24 @@ void launch_hop(const HopArgs<S, L, C> &a, int mode, bool dag, bool norm, cudaSt
             return;
         }
     }
-    // twisted mass runs on the generic kernel (hop_kernel) in every storage
-    // format; the set-up and final modes have the fast kernel in FP64, without dagger
+    // the set-up and final modes are built in FP64, without dagger
     const bool extra = std::is_same<S, F64>::value && !dag && (mode == SELF_PLAIN || mode == CLOV_SUM || mode == RESID);
-    if ((mode == HOP_CLOV || mode == SELF_CLOV || extra) && (a.tau == 0.0 || mode == SELF_PLAIN)) {
-        FastHop<S> f = make_fast(a);
-        const HopShape sh = a.fixed_shape ? HopShape{1, 1, 1, 1} : hopf_tuned<S>(f, mode, st);
-        f.gpb = sh.gpb;
-        f.minb = sh.minb;
-        f.swz = sh.swz;
-        const bool quad = is_tile_shape(sh.nr);
-        if (quad && norm && !a.red.partial_f) throw Error{LQCD_EINVAL, "tile hopping kernel: no FP32 partials"};
-        {
-            ProfScope prof(kHopNames[pi][mode], double(a.g.vh) * (nact * per_rhs + (nact ? shared : 0.0)), st);
-            hopf_launch<S>(f, sh.nr, mode, dag, norm, st);
-            LQCD_CHECK_LAUNCH();
-        }
-        if (norm) launch_partial_finish(a.red, a.ntiles, a.nrhs, a.gate_st, a.gate, st, quad);
-        return;
+    if (mode != HOP_CLOV && mode != SELF_CLOV && !extra)
+        throw Error{LQCD_EINVAL, "hopping kernel: mode not built for this precision"};
+    FastHop<S> f = make_fast(a);
+    const int kmode = a.tau != 0.0 && mode != SELF_PLAIN ? mode + TWIST : mode;
+    const HopShape sh = a.fixed_shape ? HopShape{1, 1, 1, 1} : hopf_tuned<S>(f, kmode, st);
+    f.gpb = sh.gpb;
+    f.minb = sh.minb;
+    f.swz = sh.swz;
+    const bool quad = is_tile_shape(sh.nr);
+    if (quad && norm && !a.red.partial_f) throw Error{LQCD_EINVAL, "tile hopping kernel: no FP32 partials"};
+    {
+        ProfScope prof(kHopNames[pi][mode], double(a.g.vh) * (nact * per_rhs + (nact ? shared : 0.0)), st);
+        hopf_launch<S>(f, sh.nr, kmode, dag, norm, st);
+        LQCD_CHECK_LAUNCH();
     }
-    ProfScope prof(kHopNames[pi][mode], double(a.g.vh) * (nact * per_rhs + (nact ? shared : 0.0)), st);
-    bool ok = hop_mode<S, L, C, HOP_CLOV>(a, mode, dag, norm, st) || hop_mode<S, L, C, SELF_CLOV>(a, mode, dag, norm, st);
-    if constexpr (std::is_same<S, F64>::value) {
-        ok = ok || hop_mode<S, L, C, SELF_PLAIN>(a, mode, dag, norm, st) ||
-             hop_mode<S, L, C, CLOV_SUM>(a, mode, dag, norm, st);
-        if (!ok && mode == RESID) {
-            if (dag) hop_go<S, L, C, RESID, true, true>(a, st);
-            else hop_go<S, L, C, RESID, false, true>(a, st);
-            ok = true;
-        }
-    }
-    if (!ok) throw Error{LQCD_EINVAL, "hopping kernel: mode not built for this precision"};
-    LQCD_CHECK_LAUNCH();
+    if (norm) launch_partial_finish(a.red, a.ntiles, a.nrhs, a.gate_st, a.gate, st, quad);
 }
 
 }  // namespace lqcd

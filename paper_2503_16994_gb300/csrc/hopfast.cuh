@@ -46,7 +46,7 @@ struct FastHop {
     int oy, oz, ot;              // cb offsets of one step in y, z, t
     double coef;
     double th_re[4], th_im[4];
-    double tau;                  // twisted mass of the site term (A64 and the small-batch kernel only)
+    double tau;                  // twisted mass 2 kappa mu of the site term (modes with TWIST; A64, small batches)
     int gpb;                     // groups of NR right-hand sides per block
     int minb;                    // register cap: minimum resident blocks per SM (1, 4 or 6)
     int swz;                     // tiles per super-tile in the block order (1: tile-major)
@@ -54,6 +54,7 @@ struct FastHop {
     SpinorField<S> in, self, out, b;  // b: RESID only
     LinkField<S> U;
     CloverField<S> clov;
+    CloverField<S> clov2; // twisted inverse: the C blocks (clov then holds B, see HopArgs)
     CloverField<S> site;  // CLOV_SUM with the norm: the site blocks A (FP64)
     const RhsState *gate_st;
     int gate;
@@ -509,8 +510,10 @@ __device__ __forceinline__ void half_dir_rhs(const FastHop<S> &a, const float u[
 }
 
 // one direction for all NR right-hand sides of this thread (odd: see spinor_site, of the output site)
-// SKIP: a hop whose inputs are zero in the whole warp adds nothing and is left out
-template <class S, int NR, int MU, int DIR, int SG, bool SKIP, typename R>
+// SKIP: a hop whose inputs are zero in the whole warp adds nothing and is left
+// out.  HALF: FP16 storage is projected on its halves (project_h); the twisted
+// modes project in FP32.
+template <class S, int NR, int MU, int DIR, int SG, bool SKIP, bool HALF, typename R>
 __device__ __forceinline__ void dir_f(const FastHop<S> &a, const int (&jj)[NR], unsigned on, int i, int y, int odd,
                                       bool wrap, R (&acc)[NR][24])
 {
@@ -533,7 +536,7 @@ __device__ __forceinline__ void dir_f(const FastHop<S> &a, const int (&jj)[NR], 
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
         if (!((on >> r) & 1)) continue;
-        if constexpr (S::W == 8) {
+        if constexpr (S::W == 8 && HALF) {
             __half2 w[12];
             const float sc = load_words(a.in, jj[r], y, w);
             half_dir_rhs<S, MU, DIR, SP>(a, u, w, sc, ph, acc[r]);
@@ -622,10 +625,42 @@ __device__ __forceinline__ void load_clov_block(const CloverField<S> &f, int par
     }
 }
 
-template <class S, int NR, int MODE, bool DAG, bool NORM>
+// r -= i t x (r += i t x with -t) on complex vectors of N components
+template <int N, typename R>
+__device__ __forceinline__ void sub_it(R *r, R t, const R *x)
+{
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+        r[2 * q] = fma(t, x[2 * q + 1], r[2 * q]);
+        r[2 * q + 1] = fma(-t, x[2 * q], r[2 * q + 1]);
+    }
+}
+
+// out = C v for both chirality blocks; TW: the twisted inverse (B - i s tau C)
+// v, s = +1 on the first block and -1 on the second (tau: negated for D^dag)
+template <class S, bool TW, typename R>
+__device__ __forceinline__ void clov_both(const FastHop<S> &a, int i, R tau, const R v[24], R out[24])
+{
+    R A[36];
+#pragma unroll
+    for (int blk = 0; blk < 2; ++blk) {
+        load_clov_block<S, R>(a.clov, a.parity, i, blk, A);
+        clov6(A, v + 12 * blk, out + 12 * blk);
+        if constexpr (TW) {
+            R c[12];
+            load_clov_block<S, R>(a.clov2, a.parity, i, blk, A);
+            clov6(A, v + 12 * blk, c);
+            sub_it<6>(out + 12 * blk, blk ? -tau : tau, c);
+        }
+    }
+}
+
+template <class S, int NR, int MODE_, bool DAG, bool NORM>
 __device__ __forceinline__ void hopf_group(const FastHop<S> &a, int tile, int g)
 {
     using R = typename real_of<S>::type;
+    constexpr int MODE = MODE_ % TWIST;
+    constexpr bool TW = MODE_ >= TWIST;
     int jj[NR];
     unsigned on = 0;
 #pragma unroll
@@ -659,39 +694,40 @@ __device__ __forceinline__ void hopf_group(const FastHop<S> &a, int tile, int g)
         constexpr bool SKIP = MODE == SELF_PLAIN && S::W == 2;
         {
             const bool w = x == a.L[0] - 1;
-            dir_f<S, NR, 0, +1, SG, SKIP, R>(a, jj, on, i, rowbase + ((w ? 0 : x + 1) >> 1), odd, w, acc);
+            dir_f<S, NR, 0, +1, SG, SKIP, !TW, R>(a, jj, on, i, rowbase + ((w ? 0 : x + 1) >> 1), odd, w, acc);
         }
         {
             const bool w = x == 0;
-            dir_f<S, NR, 0, -1, SG, SKIP, R>(a, jj, on, i, rowbase + ((w ? a.L[0] - 1 : x - 1) >> 1), odd, w, acc);
+            dir_f<S, NR, 0, -1, SG, SKIP, !TW, R>(a, jj, on, i, rowbase + ((w ? a.L[0] - 1 : x - 1) >> 1), odd, w, acc);
         }
         {
             const bool w = y == a.L[1] - 1;
-            dir_f<S, NR, 1, +1, SG, SKIP, R>(a, jj, on, i, i + (w ? -(a.L[1] - 1) * a.oy : a.oy), odd, w, acc);
+            dir_f<S, NR, 1, +1, SG, SKIP, !TW, R>(a, jj, on, i, i + (w ? -(a.L[1] - 1) * a.oy : a.oy), odd, w, acc);
         }
         {
             const bool w = y == 0;
-            dir_f<S, NR, 1, -1, SG, SKIP, R>(a, jj, on, i, i - (w ? -(a.L[1] - 1) * a.oy : a.oy), odd, w, acc);
+            dir_f<S, NR, 1, -1, SG, SKIP, !TW, R>(a, jj, on, i, i - (w ? -(a.L[1] - 1) * a.oy : a.oy), odd, w, acc);
         }
         {
             const bool w = z == a.L[2] - 1;
-            dir_f<S, NR, 2, +1, SG, SKIP, R>(a, jj, on, i, i + (w ? -(a.L[2] - 1) * a.oz : a.oz), odd, w, acc);
+            dir_f<S, NR, 2, +1, SG, SKIP, !TW, R>(a, jj, on, i, i + (w ? -(a.L[2] - 1) * a.oz : a.oz), odd, w, acc);
         }
         {
             const bool w = z == 0;
-            dir_f<S, NR, 2, -1, SG, SKIP, R>(a, jj, on, i, i - (w ? -(a.L[2] - 1) * a.oz : a.oz), odd, w, acc);
+            dir_f<S, NR, 2, -1, SG, SKIP, !TW, R>(a, jj, on, i, i - (w ? -(a.L[2] - 1) * a.oz : a.oz), odd, w, acc);
         }
         {
             const bool w = t == a.L[3] - 1;
-            dir_f<S, NR, 3, +1, SG, SKIP, R>(a, jj, on, i, i + (w ? -(a.L[3] - 1) * a.ot : a.ot), odd, w, acc);
+            dir_f<S, NR, 3, +1, SG, SKIP, !TW, R>(a, jj, on, i, i + (w ? -(a.L[3] - 1) * a.ot : a.ot), odd, w, acc);
         }
         {
             const bool w = t == 0;
-            dir_f<S, NR, 3, -1, SG, SKIP, R>(a, jj, on, i, i - (w ? -(a.L[3] - 1) * a.ot : a.ot), odd, w, acc);
+            dir_f<S, NR, 3, -1, SG, SKIP, !TW, R>(a, jj, on, i, i - (w ? -(a.L[3] - 1) * a.ot : a.ot), odd, w, acc);
         }
     }
     // epilogue, one right-hand side at a time
     const R coef = R(a.coef);
+    const R tau = R(DAG ? -a.tau : a.tau);
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
         if (!((on >> r) & 1)) continue;
@@ -712,19 +748,15 @@ __device__ __forceinline__ void hopf_group(const FastHop<S> &a, int tile, int g)
 #pragma unroll
                     for (int q = 0; q < 24; ++q) res[q] = sv[q];
                 } else {
-                    R A[36];
-#pragma unroll
-                    for (int blk = 0; blk < 2; ++blk) {
-                        load_clov_block<S, R>(a.clov, a.parity, i, blk, A);
-                        clov6(A, sv + 12 * blk, res + 12 * blk);
-                    }
+                    clov_both<S, TW>(a, i, tau, sv, res);
                     if constexpr (NORM) {
                         // |self + coef H in - A out|^2: the residual of the sites just solved
-                        R ao[12], t = R(0);
+                        R A[36], ao[12], t = R(0);
 #pragma unroll
                         for (int blk = 0; blk < 2; ++blk) {
                             load_clov_block<S, R>(a.site, a.parity, i, blk, A);
                             clov6(A, res + 12 * blk, ao);
+                            if constexpr (TW) sub_it<6>(ao, blk ? tau : -tau, res + 12 * blk);
 #pragma unroll
                             for (int q = 0; q < 12; ++q) {
                                 const R d = sv[12 * blk + q] - ao[q];
@@ -736,12 +768,7 @@ __device__ __forceinline__ void hopf_group(const FastHop<S> &a, int tile, int g)
                 }
             } else if constexpr (MODE == HOP_CLOV) {
                 // out = coef * C (H in)
-                R A[36];
-#pragma unroll
-                for (int blk = 0; blk < 2; ++blk) {
-                    load_clov_block<S, R>(a.clov, a.parity, i, blk, A);
-                    clov6(A, acc[r] + 12 * blk, res + 12 * blk);
-                }
+                clov_both<S, TW>(a, i, tau, acc[r], res);
 #pragma unroll
                 for (int q = 0; q < 24; ++q) res[q] *= coef;
             } else {
@@ -752,22 +779,13 @@ __device__ __forceinline__ void hopf_group(const FastHop<S> &a, int tile, int g)
 #pragma unroll
                     for (int q = 0; q < 24; ++q) sv[q] *= sc;
                 }
-                R A[36];
-#pragma unroll
-                for (int blk = 0; blk < 2; ++blk) {
-                    load_clov_block<S, R>(a.clov, a.parity, i, blk, A);
-                    clov6(A, sv + 12 * blk, res + 12 * blk);
-                }
-                if constexpr (std::is_same<S, A64>::value) {
-                    if (a.tau != 0.0) {  // + i tau g5 self
-                        const R tau = DAG ? -a.tau : a.tau;
-#pragma unroll
-                        for (int q = 0; q < 12; ++q) {
-                            const R ts = q < 6 ? tau : -tau;
-                            res[2 * q] = fma(-ts, sv[2 * q + 1], res[2 * q]);
-                            res[2 * q + 1] = fma(ts, sv[2 * q], res[2 * q + 1]);
-                        }
-                    }
+                clov_both<S, false>(a, i, tau, sv, res);
+                // + i tau g5 self
+                bool twist = TW;
+                if constexpr (std::is_same<S, A64>::value) twist = tau != R(0);
+                if (twist) {
+                    sub_it<6>(res, -tau, sv);
+                    sub_it<6>(res + 12, tau, sv + 12);
                 }
 #pragma unroll
                 for (int q = 0; q < 24; ++q) res[q] = fma(coef, acc[r][q], res[q]);
@@ -1106,14 +1124,14 @@ __device__ __forceinline__ void dir_words(const FastHop<S> &a, const float u[18]
     }
 }
 
-template <class S, int MU, int DIR, int SG>
+template <class S, int MU, int DIR, int SG, bool HALF>
 __device__ __forceinline__ void dir_p(const FastHop<S> &a, int ja, int jb, int i, int y, bool wrap, cp acc[12])
 {
     constexpr int SP = DIR > 0 ? -SG : SG;
     float u[18];
     load_link18<S, float>(a.U, DIR > 0 ? a.parity : (a.parity ^ 1), MU, DIR > 0 ? i : y, u);
     cp h[2][3], g[2][3];
-    if constexpr (S::W == 8) {
+    if constexpr (S::W == 8 && HALF) {
         __half2 wa[12], wb[12];
         const float sa = load_words(a.in, ja, y, wa), sb = load_words(a.in, jb, y, wb);
         dir_words<S, MU, DIR, SP>(a, u, wa, wb, sa, sb, wrap, acc);
@@ -1161,11 +1179,21 @@ __device__ __forceinline__ void clov6_p(const float A[36], const cp *v, cp *o)
     }
 }
 
+// r -= i t x on six components, both lanes (sub_it)
+__device__ __forceinline__ void sub_it_p(cp *r, float t, const cp *x)
+{
+#pragma unroll
+    for (int q = 0; q < 6; ++q) r[q] = cp{p_fma(bc(t), x[q].i, r[q].r), p_fma(bc(-t), x[q].r, r[q].i)};
+}
+
 // clover epilogue, store and norm partials of a pair of right-hand sides
-template <class S, int MODE, bool NORM>
+template <class S, int MODE_, bool DAG, bool NORM>
 __device__ __forceinline__ void hopp_epilogue(const FastHop<S> &a, int tile, int i, bool valid, int ja, bool on_a,
                                               int jb, bool on_b, const cp acc[12])
 {
+    constexpr int MODE = MODE_ % TWIST;
+    constexpr bool TW = MODE_ >= TWIST;
+    const float tau = float(DAG ? -a.tau : a.tau);
     double n2a = 0.0, n2b = 0.0;
     if (valid) {
         cp res[12];
@@ -1176,6 +1204,12 @@ __device__ __forceinline__ void hopp_epilogue(const FastHop<S> &a, int tile, int
             for (int blk = 0; blk < 2; ++blk) {
                 load_clov_block<S, float>(a.clov, a.parity, i, blk, A);
                 clov6_p(A, acc + 6 * blk, res + 6 * blk);
+                if constexpr (TW) {  // (B - i s tau C) v
+                    cp c[6];
+                    load_clov_block<S, float>(a.clov2, a.parity, i, blk, A);
+                    clov6_p(A, acc + 6 * blk, c);
+                    sub_it_p(res + 6 * blk, blk ? -tau : tau, c);
+                }
             }
 #pragma unroll
             for (int q = 0; q < 12; ++q) res[q] = cp{p_mul(cf, res[q].r), p_mul(cf, res[q].i)};
@@ -1191,6 +1225,7 @@ __device__ __forceinline__ void hopp_epilogue(const FastHop<S> &a, int tile, int
             for (int blk = 0; blk < 2; ++blk) {
                 load_clov_block<S, float>(a.clov, a.parity, i, blk, A);
                 clov6_p(A, sv + 6 * blk, res + 6 * blk);
+                if constexpr (TW) sub_it_p(res + 6 * blk, blk ? tau : -tau, sv + 6 * blk);  // + i s tau self
             }
 #pragma unroll
             for (int q = 0; q < 12; ++q) res[q] = cp{p_fma(cf, acc[q].r, res[q].r), p_fma(cf, acc[q].i, res[q].i)};
@@ -1235,23 +1270,23 @@ __device__ __forceinline__ void hopp_group(const FastHop<S> &a, int tile, int g)
         constexpr int SG = DAG ? -1 : 1;
         bool w;
         w = x == a.L[0] - 1;
-        dir_p<S, 0, +1, SG>(a, ja, jb, i, rowbase + ((w ? 0 : x + 1) >> 1), w, acc);
+        dir_p<S, 0, +1, SG, (MODE < TWIST)>(a, ja, jb, i, rowbase + ((w ? 0 : x + 1) >> 1), w, acc);
         w = x == 0;
-        dir_p<S, 0, -1, SG>(a, ja, jb, i, rowbase + ((w ? a.L[0] - 1 : x - 1) >> 1), w, acc);
+        dir_p<S, 0, -1, SG, (MODE < TWIST)>(a, ja, jb, i, rowbase + ((w ? a.L[0] - 1 : x - 1) >> 1), w, acc);
         w = y == a.L[1] - 1;
-        dir_p<S, 1, +1, SG>(a, ja, jb, i, i + (w ? -(a.L[1] - 1) * a.oy : a.oy), w, acc);
+        dir_p<S, 1, +1, SG, (MODE < TWIST)>(a, ja, jb, i, i + (w ? -(a.L[1] - 1) * a.oy : a.oy), w, acc);
         w = y == 0;
-        dir_p<S, 1, -1, SG>(a, ja, jb, i, i - (w ? -(a.L[1] - 1) * a.oy : a.oy), w, acc);
+        dir_p<S, 1, -1, SG, (MODE < TWIST)>(a, ja, jb, i, i - (w ? -(a.L[1] - 1) * a.oy : a.oy), w, acc);
         w = z == a.L[2] - 1;
-        dir_p<S, 2, +1, SG>(a, ja, jb, i, i + (w ? -(a.L[2] - 1) * a.oz : a.oz), w, acc);
+        dir_p<S, 2, +1, SG, (MODE < TWIST)>(a, ja, jb, i, i + (w ? -(a.L[2] - 1) * a.oz : a.oz), w, acc);
         w = z == 0;
-        dir_p<S, 2, -1, SG>(a, ja, jb, i, i - (w ? -(a.L[2] - 1) * a.oz : a.oz), w, acc);
+        dir_p<S, 2, -1, SG, (MODE < TWIST)>(a, ja, jb, i, i - (w ? -(a.L[2] - 1) * a.oz : a.oz), w, acc);
         w = t == a.L[3] - 1;
-        dir_p<S, 3, +1, SG>(a, ja, jb, i, i + (w ? -(a.L[3] - 1) * a.ot : a.ot), w, acc);
+        dir_p<S, 3, +1, SG, (MODE < TWIST)>(a, ja, jb, i, i + (w ? -(a.L[3] - 1) * a.ot : a.ot), w, acc);
         w = t == 0;
-        dir_p<S, 3, -1, SG>(a, ja, jb, i, i - (w ? -(a.L[3] - 1) * a.ot : a.ot), w, acc);
+        dir_p<S, 3, -1, SG, (MODE < TWIST)>(a, ja, jb, i, i - (w ? -(a.L[3] - 1) * a.ot : a.ot), w, acc);
     }
-    hopp_epilogue<S, MODE, NORM>(a, tile, i, valid, ja, on_a, jb, on_b, acc);
+    hopp_epilogue<S, MODE, DAG, NORM>(a, tile, i, valid, ja, on_a, jb, on_b, acc);
 }
 
 // Block b handles tile b / nbt and pair groups [(b % nbt) gpb, ... + gpb).

@@ -190,7 +190,7 @@ __device__ __forceinline__ void hops_group(const FastHop<F16> &a, int tile, int 
         stage_prologue<PD, SG, 0>(a, ja, jb, i, nb, stage);
         stage_step<0, PD, SG>(a, ja, jb, i, nb, wm, stage, acc);
     }
-    hopp_epilogue<F16, MODE, NORM>(a, tile, i, valid, ja, on_a, jb, on_b, acc);
+    hopp_epilogue<F16, MODE, DAG, NORM>(a, tile, i, valid, ja, on_a, jb, on_b, acc);
 }
 
 // bytes of dynamic shared memory per block of kBlock threads

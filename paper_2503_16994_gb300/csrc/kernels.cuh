@@ -205,7 +205,8 @@ enum HopMode : int {
     SELF_CLOV = 1,  // out = C self + coef * H in
     SELF_PLAIN = 2, // out = self + coef * H in
     CLOV_SUM = 3,   // out = C (self + coef * H in), C an inverse; its norm is |self + coef * H in - A out|^2
-    RESID = 4       // |b - (C self + coef * H in)|^2 only, nothing stored
+    RESID = 4,      // |b - (C self + coef * H in)|^2 only, nothing stored
+    TWIST = 8       // added to a mode inside the launcher: the site term with its twisted mass
 };
 
 template <class S, class L, class C>
@@ -229,29 +230,6 @@ struct HopArgs {
     bool fixed_shape = false; // true: the scalar one-RHS-per-thread shape, neither tuned nor forced by
                               // the environment (its bits do not depend on the tuner's choice)
 };
-
-template <class S, class L, class C, typename R, int MU, int SGN>
-__device__ __forceinline__ void hop_dir(const HopArgs<S, L, C> &a, int j, int i, const int x[4], spinor<R> &acc)
-{
-    constexpr int SF = -SGN;  // forward projector (1 - s g)
-    constexpr int SB = SGN;   // backward projector (1 + s g)
-    {
-        int y = cb_neighbour(a.g, x, MU, +1);
-        su3<R> U = load_link<L, R>(a.U, a.parity, MU, i);
-        spinor<R> p = load_spinor<S, R>(a.in, j, y);
-        hspinor<R> h = mul(U, project<R, MU, SF>(p));
-        if (x[MU] == a.g.L[MU] - 1) scale_h(h, cx<R>{R(a.th_re[MU]), R(a.th_im[MU])});
-        accumulate<R, MU, SF>(acc, h);
-    }
-    {
-        int y = cb_neighbour(a.g, x, MU, -1);
-        su3<R> U = load_link<L, R>(a.U, a.parity ^ 1, MU, y);
-        spinor<R> p = load_spinor<S, R>(a.in, j, y);
-        hspinor<R> h = mul_dag(U, project<R, MU, SB>(p));
-        if (x[MU] == 0) scale_h(h, cx<R>{R(a.th_re[MU]), R(-a.th_im[MU])});
-        accumulate<R, MU, SB>(acc, h);
-    }
-}
 
 template <typename R> __device__ __forceinline__ spinor<R> axpy_sp(R c, const spinor<R> &x, const spinor<R> &y)
 {
@@ -294,80 +272,6 @@ template <typename R> __device__ __forceinline__ double norm2_sp(const spinor<R>
 #pragma unroll
         for (int k = 0; k < 3; ++k) acc += norm2(x.s[s][k]);
     return double(acc);
-}
-
-template <class S, class L, class C, typename R, int MODE, bool DAG, bool NORM>
-__global__ void __launch_bounds__(128) hop_kernel(const HopArgs<S, L, C> a)
-{
-    const int j = blockIdx.x % a.nrhs;
-    const int tile = blockIdx.x / a.nrhs;
-    if (a.gate_st && a.gate_st[j].status != a.gate) return;
-    const int i = tile * blockDim.x + threadIdx.x;
-    double n2 = 0.0;
-    if (i < a.g.vh) {
-        int x[4];
-        cb_coords(a.g, a.parity, i, x);
-        spinor<R> acc;
-        zero(acc);
-        constexpr int SG = DAG ? -1 : 1;
-        hop_dir<S, L, C, R, 0, SG>(a, j, i, x, acc);
-        hop_dir<S, L, C, R, 1, SG>(a, j, i, x, acc);
-        hop_dir<S, L, C, R, 2, SG>(a, j, i, x, acc);
-        hop_dir<S, L, C, R, 3, SG>(a, j, i, x, acc);
-        const R coef = R(a.coef);
-        // twisted mass: the site term is A + i tau g5, its adjoint takes -tau
-        const R tau = R(DAG ? -a.tau : a.tau);
-        spinor<R> res;
-        if constexpr (MODE == HOP_CLOV) {
-            clover_block<R> blk[2];
-            load_clover<C, R>(a.clov, a.parity, i, blk);
-            if (tau != R(0)) {
-                clover_block<R> blk2[2];
-                load_clover<C, R>(a.clov2, a.parity, i, blk2);
-                res = twisted_inverse(blk, blk2, tau, acc);
-            } else {
-                res = clover_apply(blk, acc);
-            }
-#pragma unroll
-            for (int s = 0; s < 4; ++s)
-#pragma unroll
-                for (int k = 0; k < 3; ++k) res.s[s][k] = coef * res.s[s][k];
-        } else if constexpr (MODE == SELF_PLAIN) {
-            res = axpy_sp(coef, acc, load_spinor<S, R>(a.self, j, i));
-        } else if constexpr (MODE == CLOV_SUM) {
-            clover_block<R> blk[2];
-            load_clover<C, R>(a.clov, a.parity, i, blk);
-            const spinor<R> v = axpy_sp(coef, acc, load_spinor<S, R>(a.self, j, i));
-            if (tau != R(0)) {
-                clover_block<R> blk2[2];
-                load_clover<C, R>(a.clov2, a.parity, i, blk2);
-                res = twisted_inverse(blk, blk2, tau, v);
-            } else {
-                res = clover_apply(blk, v);
-            }
-            if constexpr (NORM) {
-                load_clover<C, R>(a.site, a.parity, i, blk);
-                spinor<R> ao = clover_apply(blk, res);
-                if (tau != R(0)) add_twist(ao, tau, res);
-                n2 = norm2_sp(axpy_sp(R(-1), ao, v));
-            }
-        } else {  // SELF_CLOV, RESID
-            clover_block<R> blk[2];
-            load_clover<C, R>(a.clov, a.parity, i, blk);
-            const spinor<R> sv = load_spinor<S, R>(a.self, j, i);
-            spinor<R> site = clover_apply(blk, sv);
-            if (tau != R(0)) add_twist(site, tau, sv);
-            res = axpy_sp(coef, acc, site);
-        }
-        if constexpr (MODE == RESID) {
-            res = axpy_sp(R(-1), res, load_spinor<S, R>(a.b, j, i));
-            n2 = norm2_sp(res);
-        } else {
-            double s2 = store_spinor<S, R>(a.out, j, i, res);
-            if (NORM && MODE != CLOV_SUM) n2 = s2;
-        }
-    }
-    if (NORM) reduce_finish(a.red, j, tile, a.ntiles, n2);
 }
 
 // ---------------------------------------------------------------------------

@@ -68,7 +68,6 @@ template <typename R> __device__ __forceinline__ R norm2(cx<R> a) { return a.re 
 // ---------------------------------------------------------------------------
 template <typename R> struct su3 { cx<R> m[3][3]; };
 template <typename R> struct spinor { cx<R> s[4][3]; };      // [spin][colour]
-template <typename R> struct hspinor { cx<R> s[2][3]; };     // projected two-spinor
 
 template <typename R> __device__ __forceinline__ void zero(spinor<R> &a)
 {
@@ -78,31 +77,7 @@ template <typename R> __device__ __forceinline__ void zero(spinor<R> &a)
         for (int c = 0; c < 3; ++c) a.s[i][c] = cx<R>{R(0), R(0)};
 }
 
-// v = U h (both spin components)
-template <typename R> __device__ __forceinline__ hspinor<R> mul(const su3<R> &U, const hspinor<R> &h)
-{
-    hspinor<R> r;
-#pragma unroll
-    for (int s = 0; s < 2; ++s)
-#pragma unroll
-        for (int a = 0; a < 3; ++a) r.s[s][a] = U.m[a][0] * h.s[s][0] + U.m[a][1] * h.s[s][1] + U.m[a][2] * h.s[s][2];
-    return r;
-}
-
-// v = U^dag h
-template <typename R> __device__ __forceinline__ hspinor<R> mul_dag(const su3<R> &U, const hspinor<R> &h)
-{
-    hspinor<R> r;
-#pragma unroll
-    for (int s = 0; s < 2; ++s)
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-            r.s[s][a] = cmul(U.m[0][a], h.s[s][0]) + cmul(U.m[1][a], h.s[s][1]) + cmul(U.m[2][a], h.s[s][2]);
-    return r;
-}
-
-// ---------------------------------------------------------------------------
-// spin projection in the chiral basis
+// The spin projection in the chiral basis,
 //
 // g_k = [[0, -i s_k], [i s_k, 0]], g_t = [[0, -1], [-1, 0]] in 2x2 spin
 // blocks (up = spins 0,1; dn = spins 2,3).  For sign s = +1 or -1,
@@ -111,70 +86,6 @@ template <typename R> __device__ __forceinline__ hspinor<R> mul_dag(const su3<R>
 // since (i s_k)^2 = -1.  So the 4-spinor is carried as the two-spinor h
 // through the colour multiplication and rebuilt afterwards.
 // i s_x (a, b) = (i b, i a); i s_y (a, b) = (b, -a); i s_z (a, b) = (i a, -i b).
-// ---------------------------------------------------------------------------
-template <typename R, int MU>
-__device__ __forceinline__ void isigma(const cx<R> a[3], const cx<R> b[3], cx<R> oa[3], cx<R> ob[3])
-{
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        if (MU == 0) { oa[c] = mul_i(b[c]); ob[c] = mul_i(a[c]); }
-        if (MU == 1) { oa[c] = b[c]; ob[c] = -a[c]; }
-        if (MU == 2) { oa[c] = mul_i(a[c]); ob[c] = -mul_i(b[c]); }
-    }
-}
-
-template <typename R, int MU, int S>
-__device__ __forceinline__ hspinor<R> project(const spinor<R> &p)
-{
-    hspinor<R> h;
-    if (MU == 3) {
-#pragma unroll
-        for (int s = 0; s < 2; ++s)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) h.s[s][c] = (S > 0) ? p.s[s][c] - p.s[2 + s][c] : p.s[s][c] + p.s[2 + s][c];
-    } else {
-        cx<R> ta[3], tb[3];
-        isigma<R, MU>(p.s[2], p.s[3], ta, tb);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            h.s[0][c] = (S > 0) ? p.s[0][c] - ta[c] : p.s[0][c] + ta[c];
-            h.s[1][c] = (S > 0) ? p.s[1][c] - tb[c] : p.s[1][c] + tb[c];
-        }
-    }
-    return h;
-}
-
-// acc += (1 + S g_mu) psi given its projection h
-template <typename R, int MU, int S>
-__device__ __forceinline__ void accumulate(spinor<R> &acc, const hspinor<R> &h)
-{
-#pragma unroll
-    for (int s = 0; s < 2; ++s)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) acc.s[s][c] = acc.s[s][c] + h.s[s][c];
-    if (MU == 3) {
-#pragma unroll
-        for (int s = 0; s < 2; ++s)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) acc.s[2 + s][c] = (S > 0) ? acc.s[2 + s][c] - h.s[s][c] : acc.s[2 + s][c] + h.s[s][c];
-    } else {
-        cx<R> ta[3], tb[3];
-        isigma<R, MU>(h.s[0], h.s[1], ta, tb);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            acc.s[2][c] = (S > 0) ? acc.s[2][c] + ta[c] : acc.s[2][c] - ta[c];
-            acc.s[3][c] = (S > 0) ? acc.s[3][c] + tb[c] : acc.s[3][c] - tb[c];
-        }
-    }
-}
-
-template <typename R> __device__ __forceinline__ void scale_h(hspinor<R> &h, cx<R> ph)
-{
-#pragma unroll
-    for (int s = 0; s < 2; ++s)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) h.s[s][c] = ph * h.s[s][c];
-}
 
 // ---------------------------------------------------------------------------
 // geometry
