@@ -58,14 +58,18 @@ WORKLOAD = {
 }
 NOMINAL_HBM_GBS = 8000.0
 # algorithmic flops per output site and RHS: hopping term 1320, clover
-# block pair 504, plus kappa scaling (hopclov, 24) or the combination with
-# the self term (selfclov, 48)
-HOP_FLOPS = {"hop_f16_hopclov": 1320 + 504 + 24, "hop_f16_selfclov": 1320 + 504 + 48}
+# block pair 504 (not in selfsum), plus kappa scaling (hopclov, 24) or the
+# combination with the self term (48)
+HOP_FLOPS = {"hop_f16_hopclov": 1320 + 504 + 24, "hop_f16_selfclov": 1320 + 504 + 48,
+             "hop_f16_addclov": 1320 + 504 + 48, "hop_f16_selfsum": 1320 + 48}
 # algorithmic bytes of the FP16 hopping kernels per output site: per active
-# RHS (spinor in + out, + self for selfclov: 52 B each) and shared by the
-# RHS of a launch (8 reconstruct-12 links of 24 B, one clover pair of 144 B)
-HOP_BYTES_PER_RHS = {"hop_f16_hopclov": 104.0, "hop_f16_selfclov": 156.0}
-HOP_BYTES_SHARED = {"hop_f16_hopclov": 336.0, "hop_f16_selfclov": 336.0}
+# RHS (spinor in + out, + self but for hopclov: 52 B each) and shared by the
+# RHS of a launch (8 reconstruct-12 links of 24 B, one clover pair of 144 B but
+# for selfsum)
+HOP_BYTES_PER_RHS = {"hop_f16_hopclov": 104.0, "hop_f16_selfclov": 156.0, "hop_f16_addclov": 156.0,
+                     "hop_f16_selfsum": 156.0}
+HOP_BYTES_SHARED = {"hop_f16_hopclov": 336.0, "hop_f16_selfclov": 336.0, "hop_f16_addclov": 336.0,
+                    "hop_f16_selfsum": 192.0}
 # DRAM bytes (read + write) per site of the FP16 12-RHS hopping kernels from
 # one ncu capture (24^3x48, 331776 sites per parity, staged paired kernel;
 # its summary is kept under profiles/): 509.4 MB for hopclov and 721.7 MB
@@ -907,7 +911,7 @@ def run_ours(args):
 
     if rank == 0:
         roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                "traffic": traffic, "kernel": "hop_f16_hopclov+selfclov",
+                "traffic": traffic, "kernel": "hop_f16_hopclov+selfsum+addclov",
                 "bytes_per_launch": hop_bytes / hop_launches if hop_launches else None,
                 "peak_source": f"{peak_kind} hbm_gbs", "frac_8TBs": achieved / NOMINAL_HBM_GBS,
                 "share": hop_ms / total_ms if total_ms else None, "launches": hop_launches,

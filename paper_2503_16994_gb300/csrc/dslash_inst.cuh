@@ -25,55 +25,66 @@ static void hopf_go(const FastHop<S> &f, cudaStream_t st)
     hopf_kernel<S, NR, MODE, DAG, NORM, 1><<<grid, kBlock, 0, st>>>(f);
 }
 
-template <class S, int NR, int MODE>
-static void hopf_mode(const FastHop<S> &f, bool dag, bool norm, cudaStream_t st)
+// What is built of each mode: HOP_CLOV and SELF_CLOV for D and D^dag without a
+// norm, SELF_SUM (D) and ADD_CLOV (D^dag) with it, as the solver uses them; in
+// FP64 also the set-up (SELF_PLAIN, no norm) and final modes (CLOV_SUM, RESID,
+// with it), for D.  The norm and the adjoint of a launch follow from the mode.
+constexpr bool mode_norm(int mode)
 {
-    if (dag) norm ? hopf_go<S, NR, MODE, true, true>(f, st) : hopf_go<S, NR, MODE, true, false>(f, st);
-    else norm ? hopf_go<S, NR, MODE, false, true>(f, st) : hopf_go<S, NR, MODE, false, false>(f, st);
+    mode %= TWIST;
+    return mode == SELF_SUM || mode == ADD_CLOV || mode == CLOV_SUM || mode == RESID;
 }
-
-template <class S, int NR, int MODE>
-static void hopf_nodag(const FastHop<S> &f, bool norm, cudaStream_t st)
+constexpr bool mode_built(int mode, bool dag, bool norm, bool f64)
 {
-    norm ? hopf_go<S, NR, MODE, false, true>(f, st) : hopf_go<S, NR, MODE, false, false>(f, st);
+    if (mode == HOP_CLOV || mode == SELF_CLOV) return !norm;
+    if (mode == SELF_SUM) return !dag && norm;
+    if (mode == ADD_CLOV) return dag && norm;
+    return f64 && !dag && norm == (mode != SELF_PLAIN);
 }
 
 template <class S, int NR>
-static void hopf_dispatch(const FastHop<S> &f, int mode, bool dag, bool norm, cudaStream_t st)
+static void hopf_dispatch(const FastHop<S> &f, int mode, bool dag, cudaStream_t st)
 {
     if constexpr (std::is_same<S, F64>::value) {
-        // the FP64 set-up and final modes of the solver (no dagger)
         switch (mode) {
-        case SELF_PLAIN: hopf_nodag<S, NR, SELF_PLAIN>(f, norm, st); return;
-        case CLOV_SUM: hopf_nodag<S, NR, CLOV_SUM>(f, norm, st); return;
-        case RESID: hopf_nodag<S, NR, RESID>(f, norm, st); return;
-        case CLOV_SUM + TWIST: hopf_nodag<S, NR, CLOV_SUM + TWIST>(f, norm, st); return;
-        case RESID + TWIST: hopf_nodag<S, NR, RESID + TWIST>(f, norm, st); return;
+        case SELF_PLAIN: hopf_go<S, NR, SELF_PLAIN, false, false>(f, st); return;
+        case CLOV_SUM: hopf_go<S, NR, CLOV_SUM, false, true>(f, st); return;
+        case RESID: hopf_go<S, NR, RESID, false, true>(f, st); return;
+        case CLOV_SUM + TWIST: hopf_go<S, NR, CLOV_SUM + TWIST, false, true>(f, st); return;
+        case RESID + TWIST: hopf_go<S, NR, RESID + TWIST, false, true>(f, st); return;
         }
     }
     if constexpr (NR == 1) {  // twisted mass: one right-hand side per thread, or the paired kernel
-        if (mode == HOP_CLOV + TWIST) {
-            hopf_mode<S, NR, HOP_CLOV + TWIST>(f, dag, norm, st);
+        switch (mode) {
+        case HOP_CLOV + TWIST:
+            dag ? hopf_go<S, NR, HOP_CLOV + TWIST, true, false>(f, st)
+                : hopf_go<S, NR, HOP_CLOV + TWIST, false, false>(f, st);
             return;
-        }
-        if (mode == SELF_CLOV + TWIST) {
-            hopf_mode<S, NR, SELF_CLOV + TWIST>(f, dag, norm, st);
+        case SELF_CLOV + TWIST:
+            dag ? hopf_go<S, NR, SELF_CLOV + TWIST, true, false>(f, st)
+                : hopf_go<S, NR, SELF_CLOV + TWIST, false, false>(f, st);
             return;
+        case SELF_SUM + TWIST: hopf_go<S, NR, SELF_SUM + TWIST, false, true>(f, st); return;
+        case ADD_CLOV + TWIST: hopf_go<S, NR, ADD_CLOV + TWIST, true, true>(f, st); return;
         }
     }
-    if (mode == HOP_CLOV) hopf_mode<S, NR, HOP_CLOV>(f, dag, norm, st);
-    else hopf_mode<S, NR, SELF_CLOV>(f, dag, norm, st);
+    switch (mode) {
+    case HOP_CLOV: dag ? hopf_go<S, NR, HOP_CLOV, true, false>(f, st) : hopf_go<S, NR, HOP_CLOV, false, false>(f, st); break;
+    case SELF_CLOV: dag ? hopf_go<S, NR, SELF_CLOV, true, false>(f, st) : hopf_go<S, NR, SELF_CLOV, false, false>(f, st); break;
+    case SELF_SUM: hopf_go<S, NR, SELF_SUM, false, true>(f, st); break;
+    default: hopf_go<S, NR, ADD_CLOV, true, true>(f, st); break;
+    }
 }
 
 // paired kernels: instantiated in hopp_f16.cu / hopp_f32.cu (own translation
 // units, so they compile in parallel with the rest)
 template <class S>
-void hopp_dispatch(const FastHop<S> &f, int mode, bool dag, bool norm, cudaStream_t st);
+void hopp_dispatch(const FastHop<S> &f, int mode, bool dag, cudaStream_t st);
 // staged paired kernel (hops_f16.cu): pd directions of cp.async copies ahead
-void hops_dispatch(const FastHop<F16> &f, int pd, int mode, bool dag, bool norm, cudaStream_t st);
+void hops_dispatch(const FastHop<F16> &f, int pd, int mode, bool dag, cudaStream_t st);
 // tile kernel (hopt_f16.cu): links, clover and neighbours prepared once per
 // 32-site tile in shared memory; pf: one direction of loads ahead
-void hopt_dispatch(const FastHop<F16> &f, bool pf, int mode, bool dag, bool norm, cudaStream_t st);
+void hopt_dispatch(const FastHop<F16> &f, bool pf, int mode, bool dag, cudaStream_t st);
 
 template <class S, int MODE, bool DAG, bool NORM>
 static void hopq_go(const FastHop<S> &f, int pf, cudaStream_t st)
@@ -85,14 +96,13 @@ static void hopq_go(const FastHop<S> &f, int pf, cudaStream_t st)
 }
 
 template <class S>
-static void hopq_dispatch(const FastHop<S> &f, int pf, int mode, bool dag, bool norm, cudaStream_t st)
+static void hopq_dispatch(const FastHop<S> &f, int pf, int mode, bool dag, cudaStream_t st)
 {
-    if (mode == HOP_CLOV) {
-        if (dag) norm ? hopq_go<S, HOP_CLOV, true, true>(f, pf, st) : hopq_go<S, HOP_CLOV, true, false>(f, pf, st);
-        else norm ? hopq_go<S, HOP_CLOV, false, true>(f, pf, st) : hopq_go<S, HOP_CLOV, false, false>(f, pf, st);
-    } else {
-        if (dag) norm ? hopq_go<S, SELF_CLOV, true, true>(f, pf, st) : hopq_go<S, SELF_CLOV, true, false>(f, pf, st);
-        else norm ? hopq_go<S, SELF_CLOV, false, true>(f, pf, st) : hopq_go<S, SELF_CLOV, false, false>(f, pf, st);
+    switch (mode) {
+    case HOP_CLOV: dag ? hopq_go<S, HOP_CLOV, true, false>(f, pf, st) : hopq_go<S, HOP_CLOV, false, false>(f, pf, st); break;
+    case SELF_CLOV: dag ? hopq_go<S, SELF_CLOV, true, false>(f, pf, st) : hopq_go<S, SELF_CLOV, false, false>(f, pf, st); break;
+    case SELF_SUM: hopq_go<S, SELF_SUM, false, true>(f, pf, st); break;
+    default: hopq_go<S, ADD_CLOV, true, true>(f, pf, st); break;
     }
 }
 
@@ -107,43 +117,43 @@ static void hopq_dispatch(const FastHop<S> &f, int pf, int mode, bool dag, bool 
 constexpr bool is_tile_shape(int nr) { return nr == 20 || nr == 21; }
 
 template <class S>
-static void hopf_launch(const FastHop<S> &f, int nr, int mode, bool dag, bool norm, cudaStream_t st)
+static void hopf_launch(const FastHop<S> &f, int nr, int mode, bool dag, cudaStream_t st)
 {
     if constexpr (std::is_same<S, F16>::value) {
         if (is_tile_shape(nr)) {
-            hopt_dispatch(f, nr == 21, mode, dag, norm, st);
+            hopt_dispatch(f, nr == 21, mode, dag, st);
             return;
         }
         if (nr >= 12) {
-            hops_dispatch(f, nr - 10, mode, dag, norm, st);
+            hops_dispatch(f, nr - 10, mode, dag, st);
             return;
         }
     }
     if constexpr (!std::is_same<S, F64>::value) {
         if (nr == 0) {
-            hopp_dispatch<S>(f, mode, dag, norm, st);
+            hopp_dispatch<S>(f, mode, dag, st);
             return;
         }
         if (nr < 0) {
-            hopq_dispatch<S>(f, -nr, mode, dag, norm, st);
+            hopq_dispatch<S>(f, -nr, mode, dag, st);
             return;
         }
     }
     if constexpr (std::is_same<S, F64>::value) {
-        hopf_dispatch<S, 1>(f, mode, dag, norm, st);
+        hopf_dispatch<S, 1>(f, mode, dag, st);
     } else {
         switch (nr) {
-        case 1: hopf_dispatch<S, 1>(f, mode, dag, norm, st); break;
-        case 2: hopf_dispatch<S, 2>(f, mode, dag, norm, st); break;
-        default: hopf_dispatch<S, 3>(f, mode, dag, norm, st); break;
+        case 1: hopf_dispatch<S, 1>(f, mode, dag, st); break;
+        case 2: hopf_dispatch<S, 2>(f, mode, dag, st); break;
+        default: hopf_dispatch<S, 3>(f, mode, dag, st); break;
         }
     }
 }
 
 // Autotuned shape: right-hand sides per thread (NR) and groups of NR per
 // block (GPB), keyed by (sites, nrhs, format, mode).  The first launch of a
-// key times the candidates (no reductions, same stream and buffers: every
-// candidate writes the output the real launch then overwrites) and keeps
+// key times the candidates (same stream and buffers: every candidate writes the
+// output and partial sums the real launch then overwrites) and keeps
 // the fastest.  LQCD_HOP_NR / LQCD_HOP_GPB force a value.
 struct HopShape {
     int nr, gpb, minb, swz;
@@ -154,7 +164,7 @@ struct HopShape {
 template <class S>
 static HopShape hopf_tuned(FastHop<S> f, int mode, cudaStream_t st)
 {
-    const bool tw = mode >= TWIST;
+    const bool tw = mode >= TWIST, dag = mode % TWIST == ADD_CLOV;  // the adjoint where only that is built
     static std::mutex mu;
     static std::map<std::tuple<int, int, int, int>, HopShape> table;
     const char *env_nr = std::getenv("LQCD_HOP_NR");
@@ -245,11 +255,11 @@ static HopShape hopf_tuned(FastHop<S> f, int mode, cudaStream_t st)
         f.gpb = c.gpb;
         f.minb = c.minb;
         f.swz = c.swz;
-        hopf_launch<S>(f, c.nr, mode, false, false, st);  // warm-up
+        hopf_launch<S>(f, c.nr, mode, dag, st);  // warm-up
         float ms_min = 1e30f;
         for (int rep = 0; rep < 2; ++rep) {
             LQCD_CUDA(cudaEventRecord(e0, st));
-            hopf_launch<S>(f, c.nr, mode, false, false, st);
+            hopf_launch<S>(f, c.nr, mode, dag, st);
             LQCD_CUDA(cudaEventRecord(e1, st));
             LQCD_CUDA(cudaEventSynchronize(e1));
             float ms = 0.f;
@@ -318,31 +328,32 @@ static FastHop<S> make_fast(const HopArgs<S, S, S> &a)
     return f;
 }
 
-// the small-lattice FP64 kernel (hopd.cuh); the norm's partials are per block of kSplitSites sites
-template <int MODE, bool NORM>
-static void hopd_go(const FastHop<F64> &f, CloverField<F64> clov2, bool dag, cudaStream_t st)
+// the small-batch FP64 kernel (hopd.cuh); the norm's partials are per block of kSplitSites sites
+template <int MODE, bool DAG>
+static void hopd_go(const FastHop<F64> &f, CloverField<F64> clov2, cudaStream_t st)
 {
     const unsigned grid = unsigned(split_blocks(f.vh) * f.nrhs);
-    if (dag) launch_pdl(hopd_kernel<F64, MODE, true, NORM>, dim3(grid), 128, 0, st, f, clov2);
-    else launch_pdl(hopd_kernel<F64, MODE, false, NORM>, dim3(grid), 128, 0, st, f, clov2);
+    launch_pdl(hopd_kernel<F64, MODE, DAG, mode_norm(MODE)>, dim3(grid), 128, 0, st, f, clov2);
 }
 
-template <bool NORM>
 static void hopd_dispatch(const FastHop<F64> &f, CloverField<F64> clov2, int mode, bool dag, cudaStream_t st)
 {
     switch (mode) {
-    case HOP_CLOV: hopd_go<HOP_CLOV, NORM>(f, clov2, dag, st); break;
-    case SELF_CLOV: hopd_go<SELF_CLOV, NORM>(f, clov2, dag, st); break;
-    case SELF_PLAIN: hopd_go<SELF_PLAIN, NORM>(f, clov2, dag, st); break;
-    case CLOV_SUM: hopd_go<CLOV_SUM, NORM>(f, clov2, dag, st); break;
-    default: hopd_go<RESID, NORM>(f, clov2, dag, st); break;
+    case HOP_CLOV: dag ? hopd_go<HOP_CLOV, true>(f, clov2, st) : hopd_go<HOP_CLOV, false>(f, clov2, st); break;
+    case SELF_CLOV: dag ? hopd_go<SELF_CLOV, true>(f, clov2, st) : hopd_go<SELF_CLOV, false>(f, clov2, st); break;
+    case SELF_PLAIN: hopd_go<SELF_PLAIN, false>(f, clov2, st); break;
+    case SELF_SUM: hopd_go<SELF_SUM, false>(f, clov2, st); break;
+    case ADD_CLOV: hopd_go<ADD_CLOV, true>(f, clov2, st); break;
+    case CLOV_SUM: hopd_go<CLOV_SUM, false>(f, clov2, st); break;
+    default: hopd_go<RESID, false>(f, clov2, st); break;
     }
 }
 
-static const char *const kHopNames[3][5] = {
-    {"hop_f64_hopclov", "hop_f64_selfclov", "hop_f64_self", "hop_f64_clovsum", "hop_f64_resid"},
-    {"hop_f32_hopclov", "hop_f32_selfclov", "hop_f32_self", "hop_f32_clovsum", "hop_f32_resid"},
-    {"hop_f16_hopclov", "hop_f16_selfclov", "hop_f16_self", "hop_f16_clovsum", "hop_f16_resid"}};
+static const char *const kHopNames[3][7] = {
+    {"hop_f64_hopclov", "hop_f64_selfclov", "hop_f64_self", "hop_f64_clovsum", "hop_f64_resid", "hop_f64_addclov",
+     "hop_f64_selfsum"},
+    {"hop_f32_hopclov", "hop_f32_selfclov", "", "", "", "hop_f32_addclov", "hop_f32_selfsum"},
+    {"hop_f16_hopclov", "hop_f16_selfclov", "", "", "", "hop_f16_addclov", "hop_f16_selfsum"}};
 
 template <class S, class L, class C>
 void launch_hop(const HopArgs<S, L, C> &a, int mode, bool dag, bool norm, cudaStream_t st)
@@ -353,25 +364,22 @@ void launch_hop(const HopArgs<S, L, C> &a, int mode, bool dag, bool norm, cudaSt
     const int nact = a.nactive >= 0 ? std::min(a.nactive, a.nrhs) : a.nrhs;  // RHS that pass the gate
     double per_rhs = sb + (mode == RESID ? 0.0 : sb) + (mode == HOP_CLOV ? 0.0 : sb) + (mode == RESID ? sb : 0.0);
     // the twisted inverse reads two Hermitian block pairs (B and C)
-    const bool twinv = a.tau != 0.0 && (mode == HOP_CLOV || mode == CLOV_SUM);
-    double shared = 8.0 * link_bytes<L>() + (mode == SELF_PLAIN ? 0.0 : (twinv ? 2.0 : 1.0) * clover_bytes<C>());
+    const bool twinv = a.tau != 0.0 && (mode == HOP_CLOV || mode == CLOV_SUM || mode == ADD_CLOV);
+    double shared = 8.0 * link_bytes<L>() + (mode == SELF_PLAIN || mode == SELF_SUM ? 0.0 : (twinv ? 2.0 : 1.0) * clover_bytes<C>());
     const int pi = S::W == 2 ? 0 : (S::W == 4 ? 1 : 2);
+    if (!mode_built(mode, dag, norm, std::is_same<S, F64>::value))
+        throw Error{LQCD_EINVAL, "hopping kernel: mode not built for this precision"};
     if constexpr (std::is_same<S, F64>::value) {
         if (split_hop(a.g.vh, a.nrhs)) {
             {
                 ProfScope prof(kHopNames[pi][mode], double(a.g.vh) * (nact * per_rhs + (nact ? shared : 0.0)), st);
-                if (norm) hopd_dispatch<true>(make_fast(a), a.clov2, mode, dag, st);
-                else hopd_dispatch<false>(make_fast(a), a.clov2, mode, dag, st);
+                hopd_dispatch(make_fast(a), a.clov2, mode, dag, st);
                 LQCD_CHECK_LAUNCH();
             }
             if (norm) launch_partial_finish(a.red, split_blocks(a.g.vh), a.nrhs, a.gate_st, a.gate, st);
             return;
         }
     }
-    // the set-up and final modes are built in FP64, without dagger
-    const bool extra = std::is_same<S, F64>::value && !dag && (mode == SELF_PLAIN || mode == CLOV_SUM || mode == RESID);
-    if (mode != HOP_CLOV && mode != SELF_CLOV && !extra)
-        throw Error{LQCD_EINVAL, "hopping kernel: mode not built for this precision"};
     FastHop<S> f = make_fast(a);
     const int kmode = a.tau != 0.0 && mode != SELF_PLAIN ? mode + TWIST : mode;
     const HopShape sh = a.fixed_shape ? HopShape{1, 1, 1, 1} : hopf_tuned<S>(f, kmode, st);
@@ -382,7 +390,7 @@ void launch_hop(const HopArgs<S, L, C> &a, int mode, bool dag, bool norm, cudaSt
     if (quad && norm && !a.red.partial_f) throw Error{LQCD_EINVAL, "tile hopping kernel: no FP32 partials"};
     {
         ProfScope prof(kHopNames[pi][mode], double(a.g.vh) * (nact * per_rhs + (nact ? shared : 0.0)), st);
-        hopf_launch<S>(f, sh.nr, kmode, dag, norm, st);
+        hopf_launch<S>(f, sh.nr, kmode, dag, st);
         LQCD_CHECK_LAUNCH();
     }
     if (norm) launch_partial_finish(a.red, a.ntiles, a.nrhs, a.gate_st, a.gate, st, quad);

@@ -93,8 +93,9 @@ __global__ void __launch_bounds__(128) hopd_kernel(const FastHop<S> a, const Clo
     const int wi = min(tile * kSplitSites + wsite, a.vh - 1);
     const bool wvalid = worker && tile * kSplitSites + wsite < a.vh;
     // the rows of the clover block are on their way while the hops run
-    constexpr bool CLOV = MODE != SELF_PLAIN;
-    constexpr bool INV = MODE == HOP_CLOV || MODE == CLOV_SUM;  // the block is an inverse: twisted by B and C
+    constexpr bool PLAIN = MODE == SELF_PLAIN || MODE == SELF_SUM, CLOV = !PLAIN;
+    // the block is an inverse: twisted by B and C
+    constexpr bool INV = MODE == HOP_CLOV || MODE == CLOV_SUM || MODE == ADD_CLOV;
     CloverRow A, A2, As;
     if (CLOV && worker) {
         load_clover_row(a.clov, parity, wi, comp / 6, comp % 6, A);
@@ -186,7 +187,7 @@ __global__ void __launch_bounds__(128) hopd_kernel(const FastHop<S> a, const Clo
     if (INV) {  // the block acts on H, or on self + coef H
         if (worker)
             vec[comp][wsite] =
-                MODE == HOP_CLOV ? H : make_double2(fma(coef, H.x, self.x), fma(coef, H.y, self.y));
+                MODE != CLOV_SUM ? H : make_double2(fma(coef, H.x, self.x), fma(coef, H.y, self.y));
         __syncthreads();
     }
     double n2 = 0.0;
@@ -204,7 +205,8 @@ __global__ void __launch_bounds__(128) hopd_kernel(const FastHop<S> a, const Clo
                 res.y = fma(-ts, c.x, res.y);
             }
             if (MODE == HOP_CLOV) res = make_double2(coef * res.x, coef * res.y);
-        } else if (MODE == SELF_PLAIN) {
+            if (MODE == ADD_CLOV) res = make_double2(fma(coef, res.x, self.x), fma(coef, res.y, self.y));
+        } else if (PLAIN) {
             res = make_double2(fma(coef, H.x, self.x), fma(coef, H.y, self.y));
         } else {
             res = clover_row(A, v, kSplitSites, r);

@@ -734,7 +734,7 @@ __device__ __forceinline__ void hopf_group(const FastHop<S> &a, int tile, int g)
         double n2 = 0.0;
         if (valid) {
             R res[24];
-            if constexpr (MODE == SELF_PLAIN || MODE == CLOV_SUM) {
+            if constexpr (MODE == SELF_PLAIN || MODE == SELF_SUM || MODE == CLOV_SUM) {
                 // self + coef H in, then (CLOV_SUM) times C
                 R sv[24];
                 const R sc = load_raw<S, R>(a.self, jj[r], spinor_site<S>(i, odd), sv);
@@ -744,7 +744,7 @@ __device__ __forceinline__ void hopf_group(const FastHop<S> &a, int tile, int g)
                 }
 #pragma unroll
                 for (int q = 0; q < 24; ++q) sv[q] = fma(coef, acc[r][q], sv[q]);
-                if constexpr (MODE == SELF_PLAIN) {
+                if constexpr (MODE != CLOV_SUM) {
 #pragma unroll
                     for (int q = 0; q < 24; ++q) res[q] = sv[q];
                 } else {
@@ -771,6 +771,17 @@ __device__ __forceinline__ void hopf_group(const FastHop<S> &a, int tile, int g)
                 clov_both<S, TW>(a, i, tau, acc[r], res);
 #pragma unroll
                 for (int q = 0; q < 24; ++q) res[q] *= coef;
+            } else if constexpr (MODE == ADD_CLOV) {
+                // out = self + coef * C (H in)
+                clov_both<S, TW>(a, i, tau, acc[r], res);
+                R sv[24];
+                const R sc = load_raw<S, R>(a.self, jj[r], i, sv);
+                if constexpr (S::W == 8) {
+#pragma unroll
+                    for (int q = 0; q < 24; ++q) sv[q] *= sc;
+                }
+#pragma unroll
+                for (int q = 0; q < 24; ++q) res[q] = fma(coef, res[q], sv[q]);
             } else {
                 // out = C self + coef * H in
                 R sv[24];
@@ -1198,7 +1209,18 @@ __device__ __forceinline__ void hopp_epilogue(const FastHop<S> &a, int tile, int
     if (valid) {
         cp res[12];
         const float2 cf = bc(float(a.coef));
-        if constexpr (MODE == HOP_CLOV) {
+        cp sv[12];
+        if constexpr (MODE != HOP_CLOV) {
+            const float2 sc = load_pair<S>(a.self, ja, jb, i, sv);
+            if constexpr (S::W == 8) {
+#pragma unroll
+                for (int q = 0; q < 12; ++q) sv[q] = cp{p_mul(sv[q].r, sc), p_mul(sv[q].i, sc)};
+            }
+        }
+        if constexpr (MODE == SELF_SUM) {
+#pragma unroll
+            for (int q = 0; q < 12; ++q) res[q] = cp{p_fma(cf, acc[q].r, sv[q].r), p_fma(cf, acc[q].i, sv[q].i)};
+        } else if constexpr (MODE == HOP_CLOV || MODE == ADD_CLOV) {
             float A[36];
 #pragma unroll
             for (int blk = 0; blk < 2; ++blk) {
@@ -1212,14 +1234,11 @@ __device__ __forceinline__ void hopp_epilogue(const FastHop<S> &a, int tile, int
                 }
             }
 #pragma unroll
-            for (int q = 0; q < 12; ++q) res[q] = cp{p_mul(cf, res[q].r), p_mul(cf, res[q].i)};
-        } else {
-            cp sv[12];
-            const float2 sc = load_pair<S>(a.self, ja, jb, i, sv);
-            if constexpr (S::W == 8) {
-#pragma unroll
-                for (int q = 0; q < 12; ++q) sv[q] = cp{p_mul(sv[q].r, sc), p_mul(sv[q].i, sc)};
+            for (int q = 0; q < 12; ++q) {
+                if constexpr (MODE == HOP_CLOV) res[q] = cp{p_mul(cf, res[q].r), p_mul(cf, res[q].i)};
+                else res[q] = cp{p_fma(cf, res[q].r, sv[q].r), p_fma(cf, res[q].i, sv[q].i)};
             }
+        } else {
             float A[36];
 #pragma unroll
             for (int blk = 0; blk < 2; ++blk) {
@@ -1514,32 +1533,31 @@ __device__ __forceinline__ void hopq_item(const FastHop<S> &a, int tile, int j)
             phase_dirs<S, 4, 2, SG>(a, j, i, nb, wm, acc);
             phase_dirs<S, 6, 2, SG>(a, j, i, nb, wm, acc);
         }
-        float res[24];
+        float res[24], sv[24];
         const float coef = float(a.coef);
-        if constexpr (MODE == HOP_CLOV) {
-            float A[36];
-#pragma unroll
-            for (int blk = 0; blk < 2; ++blk) {
-                load_clov_block<S, float>(a.clov, a.parity, i, blk, A);
-                clov6(A, acc + 12 * blk, res + 12 * blk);
-            }
-#pragma unroll
-            for (int q = 0; q < 24; ++q) res[q] *= coef;
-        } else {
-            float sv[24];
+        if constexpr (MODE != HOP_CLOV) {
             const float sc = load_raw<S, float>(a.self, j, i, sv);
             if constexpr (S::W == 8) {
 #pragma unroll
                 for (int q = 0; q < 24; ++q) sv[q] *= sc;
             }
+        }
+        if constexpr (MODE == SELF_SUM) {
+#pragma unroll
+            for (int q = 0; q < 24; ++q) res[q] = fmaf(coef, acc[q], sv[q]);
+        } else {
             float A[36];
 #pragma unroll
             for (int blk = 0; blk < 2; ++blk) {
                 load_clov_block<S, float>(a.clov, a.parity, i, blk, A);
-                clov6(A, sv + 12 * blk, res + 12 * blk);
+                clov6(A, (MODE == SELF_CLOV ? sv : acc) + 12 * blk, res + 12 * blk);
             }
 #pragma unroll
-            for (int q = 0; q < 24; ++q) res[q] = fmaf(coef, acc[q], res[q]);
+            for (int q = 0; q < 24; ++q) {
+                if constexpr (MODE == HOP_CLOV) res[q] *= coef;
+                else if constexpr (MODE == ADD_CLOV) res[q] = fmaf(coef, res[q], sv[q]);
+                else res[q] = fmaf(coef, acc[q], res[q]);
+            }
         }
         n2 = store_raw<S, float>(a.out, j, i, res);
     }

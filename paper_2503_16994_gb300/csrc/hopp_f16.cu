@@ -2,5 +2,5 @@
 #include "hopp_inst.cuh"
 
 namespace lqcd {
-template void hopp_dispatch<F16>(const FastHop<F16> &, int, bool, bool, cudaStream_t);
+template void hopp_dispatch<F16>(const FastHop<F16> &, int, bool, cudaStream_t);
 }  // namespace lqcd

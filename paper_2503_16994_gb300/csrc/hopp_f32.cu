@@ -2,5 +2,5 @@
 #include "hopp_inst.cuh"
 
 namespace lqcd {
-template void hopp_dispatch<F32>(const FastHop<F32> &, int, bool, bool, cudaStream_t);
+template void hopp_dispatch<F32>(const FastHop<F32> &, int, bool, cudaStream_t);
 }  // namespace lqcd

@@ -19,21 +19,22 @@ static void hopp_go(const FastHop<S> &f, cudaStream_t st)
         hopp_kernel<S, MODE, DAG, NORM, 1><<<grid, kBlock, 0, st>>>(f);
 }
 
-template <class S, int MODE>
-static void hopp_mode(const FastHop<S> &f, bool dag, bool norm, cudaStream_t st)
-{
-    if (dag) norm ? hopp_go<S, MODE, true, true>(f, st) : hopp_go<S, MODE, true, false>(f, st);
-    else norm ? hopp_go<S, MODE, false, true>(f, st) : hopp_go<S, MODE, false, false>(f, st);
-}
-
 template <class S>
-void hopp_dispatch(const FastHop<S> &f, int mode, bool dag, bool norm, cudaStream_t st)
+void hopp_dispatch(const FastHop<S> &f, int mode, bool dag, cudaStream_t st)
 {
     switch (mode) {
-    case HOP_CLOV: hopp_mode<S, HOP_CLOV>(f, dag, norm, st); break;
-    case SELF_CLOV: hopp_mode<S, SELF_CLOV>(f, dag, norm, st); break;
-    case HOP_CLOV + TWIST: hopp_mode<S, HOP_CLOV + TWIST>(f, dag, norm, st); break;
-    default: hopp_mode<S, SELF_CLOV + TWIST>(f, dag, norm, st); break;
+    case HOP_CLOV: dag ? hopp_go<S, HOP_CLOV, true, false>(f, st) : hopp_go<S, HOP_CLOV, false, false>(f, st); break;
+    case SELF_CLOV: dag ? hopp_go<S, SELF_CLOV, true, false>(f, st) : hopp_go<S, SELF_CLOV, false, false>(f, st); break;
+    case SELF_SUM: hopp_go<S, SELF_SUM, false, true>(f, st); break;
+    case ADD_CLOV: hopp_go<S, ADD_CLOV, true, true>(f, st); break;
+    case HOP_CLOV + TWIST:
+        dag ? hopp_go<S, HOP_CLOV + TWIST, true, false>(f, st) : hopp_go<S, HOP_CLOV + TWIST, false, false>(f, st);
+        break;
+    case SELF_CLOV + TWIST:
+        dag ? hopp_go<S, SELF_CLOV + TWIST, true, false>(f, st) : hopp_go<S, SELF_CLOV + TWIST, false, false>(f, st);
+        break;
+    case SELF_SUM + TWIST: hopp_go<S, SELF_SUM + TWIST, false, true>(f, st); break;
+    default: hopp_go<S, ADD_CLOV + TWIST, true, true>(f, st); break;
     }
 }
 

@@ -43,14 +43,13 @@ static void hops_go(const FastHop<F16> &f, int pd, cudaStream_t st)
     else hops_launch<MODE, DAG, NORM, 3, 2>(f, grid, st);
 }
 
-void hops_dispatch(const FastHop<F16> &f, int pd, int mode, bool dag, bool norm, cudaStream_t st)
+void hops_dispatch(const FastHop<F16> &f, int pd, int mode, bool dag, cudaStream_t st)
 {
-    if (mode == HOP_CLOV) {
-        if (dag) norm ? hops_go<HOP_CLOV, true, true>(f, pd, st) : hops_go<HOP_CLOV, true, false>(f, pd, st);
-        else norm ? hops_go<HOP_CLOV, false, true>(f, pd, st) : hops_go<HOP_CLOV, false, false>(f, pd, st);
-    } else {
-        if (dag) norm ? hops_go<SELF_CLOV, true, true>(f, pd, st) : hops_go<SELF_CLOV, true, false>(f, pd, st);
-        else norm ? hops_go<SELF_CLOV, false, true>(f, pd, st) : hops_go<SELF_CLOV, false, false>(f, pd, st);
+    switch (mode) {
+    case HOP_CLOV: dag ? hops_go<HOP_CLOV, true, false>(f, pd, st) : hops_go<HOP_CLOV, false, false>(f, pd, st); break;
+    case SELF_CLOV: dag ? hops_go<SELF_CLOV, true, false>(f, pd, st) : hops_go<SELF_CLOV, false, false>(f, pd, st); break;
+    case SELF_SUM: hops_go<SELF_SUM, false, true>(f, pd, st); break;
+    default: hops_go<ADD_CLOV, true, true>(f, pd, st); break;
     }
 }
 

@@ -288,38 +288,27 @@ __global__ void __launch_bounds__(kTileSites * kTileMaxPairs, MINB) hopt_kernel(
     if (valid) {
         cp res[12];
         const float2 cf = bc(float(a.coef));
-        if constexpr (MODE == HOP_CLOV) {
+        // the arithmetic of hopp_epilogue (load_pair, scale, clov6_p, fma)
+        cp sv[12];
+        if constexpr (MODE != HOP_CLOV) {
+            const float2 sc = load_pair<F16>(a.self, ja, jb, i, sv);
 #pragma unroll
-            for (int blk = 0; blk < 2; ++blk) clov6_tile(&sh.c[18 * blk][s], acc + 6 * blk, res + 6 * blk);
+            for (int q = 0; q < 12; ++q) sv[q] = cp{p_mul(sv[q].r, sc), p_mul(sv[q].i, sc)};
+        }
+        if constexpr (MODE == SELF_SUM) {
 #pragma unroll
-            for (int q = 0; q < 12; ++q) res[q] = cp{p_mul(cf, res[q].r), p_mul(cf, res[q].i)};
+            for (int q = 0; q < 12; ++q) res[q] = cp{p_fma(cf, acc[q].r, sv[q].r), p_fma(cf, acc[q].i, sv[q].i)};
         } else {
-            // the arithmetic of hopp_epilogue (load_pair, scale, clov6_p, fma), one clover block at a time
-            const long st = a.self.stride;
-            const uint4 *pa = a.self.p + (long)ja * 3 * st + i;
-            const uint4 *pb = a.self.p + (long)jb * 3 * st + i;
-            uint4 wsa[3], wsb[3];
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                wsa[k] = __ldg(pa + k * st);
-                wsb[k] = __ldg(pb + k * st);
+            for (int blk = 0; blk < 2; ++blk)
+                clov6_tile(&sh.c[18 * blk][s], (MODE == SELF_CLOV ? sv : acc) + 6 * blk, res + 6 * blk);
+#pragma unroll
+            for (int q = 0; q < 12; ++q) {
+                if constexpr (MODE == HOP_CLOV) res[q] = cp{p_mul(cf, res[q].r), p_mul(cf, res[q].i)};
+                else if constexpr (MODE == ADD_CLOV)
+                    res[q] = cp{p_fma(cf, res[q].r, sv[q].r), p_fma(cf, res[q].i, sv[q].i)};
+                else res[q] = cp{p_fma(cf, acc[q].r, res[q].r), p_fma(cf, acc[q].i, res[q].i)};
             }
-            const float2 sc = make_float2(__ldg(a.self.scale + (long)ja * st + i), __ldg(a.self.scale + (long)jb * st + i));
-#pragma unroll
-            for (int blk = 0; blk < 2; ++blk) {
-                cp sv[6];
-#pragma unroll
-                for (int r = 0; r < 6; ++r) {
-                    const int q = 6 * blk + r;  // complex component 0..11: word q / 4, half2 q % 4
-                    const __half2 ha = reinterpret_cast<const __half2 *>(&wsa[q / 4])[q % 4];
-                    const __half2 hb = reinterpret_cast<const __half2 *>(&wsb[q / 4])[q % 4];
-                    const cp v{__half22float2(__lows2half2(ha, hb)), __half22float2(__highs2half2(ha, hb))};
-                    sv[r] = cp{p_mul(v.r, sc), p_mul(v.i, sc)};
-                }
-                clov6_tile(&sh.c[18 * blk][s], sv, res + 6 * blk);
-            }
-#pragma unroll
-            for (int q = 0; q < 12; ++q) res[q] = cp{p_fma(cf, acc[q].r, res[q].r), p_fma(cf, acc[q].i, res[q].i)};
         }
         float va[24], vb[24];
 #pragma unroll

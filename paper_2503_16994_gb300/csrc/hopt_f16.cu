@@ -46,14 +46,13 @@ static void hopt_go(const FastHop<F16> &f, bool pf, cudaStream_t st)
 
 // gpb: pairs of right-hand sides (warps) per block; pf: spinor words staged
 // two directions ahead instead of one (registers capped for 2 blocks per SM)
-void hopt_dispatch(const FastHop<F16> &f, bool pf, int mode, bool dag, bool norm, cudaStream_t st)
+void hopt_dispatch(const FastHop<F16> &f, bool pf, int mode, bool dag, cudaStream_t st)
 {
-    if (mode == HOP_CLOV) {
-        if (dag) norm ? hopt_go<HOP_CLOV, true, true>(f, pf, st) : hopt_go<HOP_CLOV, true, false>(f, pf, st);
-        else norm ? hopt_go<HOP_CLOV, false, true>(f, pf, st) : hopt_go<HOP_CLOV, false, false>(f, pf, st);
-    } else {
-        if (dag) norm ? hopt_go<SELF_CLOV, true, true>(f, pf, st) : hopt_go<SELF_CLOV, true, false>(f, pf, st);
-        else norm ? hopt_go<SELF_CLOV, false, true>(f, pf, st) : hopt_go<SELF_CLOV, false, false>(f, pf, st);
+    switch (mode) {
+    case HOP_CLOV: dag ? hopt_go<HOP_CLOV, true, false>(f, pf, st) : hopt_go<HOP_CLOV, false, false>(f, pf, st); break;
+    case SELF_CLOV: dag ? hopt_go<SELF_CLOV, true, false>(f, pf, st) : hopt_go<SELF_CLOV, false, false>(f, pf, st); break;
+    case SELF_SUM: hopt_go<SELF_SUM, false, true>(f, pf, st); break;
+    default: hopt_go<ADD_CLOV, true, true>(f, pf, st); break;
     }
 }
 

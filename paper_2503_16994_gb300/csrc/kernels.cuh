@@ -206,6 +206,8 @@ enum HopMode : int {
     SELF_PLAIN = 2, // out = self + coef * H in
     CLOV_SUM = 3,   // out = C (self + coef * H in), C an inverse; its norm is |self + coef * H in - A out|^2
     RESID = 4,      // |b - (C self + coef * H in)|^2 only, nothing stored
+    ADD_CLOV = 5,   // out = self + coef * C (H in)
+    SELF_SUM = 6,   // out = self + coef * H in (the solver's; SELF_PLAIN is its set-up's)
     TWIST = 8       // added to a mode inside the launcher: the site term with its twisted mass
 };
 
@@ -315,12 +317,6 @@ template <typename R> __device__ __forceinline__ R alpha_of(const RhsState &s)
     if constexpr (std::is_same<R, float>::value) return s.alpha_f;
     else return s.alpha;
 }
-template <typename R> __device__ __forceinline__ R beta_of(const RhsState &s)
-{
-    if constexpr (std::is_same<R, float>::value) return s.beta_f;
-    else return s.beta;
-}
-
 template <class W, class E>
 __global__ void __launch_bounds__(128) cg_er_update(VecArgs v, SpinorField<W> p, SpinorField<W> w, SpinorField<W> r,
                                                     SpinorField<E> e)
@@ -339,19 +335,6 @@ __global__ void __launch_bounds__(128) cg_er_update(VecArgs v, SpinorField<W> p,
         n2 = store_spinor<W, R>(r, j, i, axpy_sp(-al, wv, rv));
     }
     reduce_finish(v.red, j, tile, v.ntiles, n2);
-}
-
-// p = z + beta p
-template <class W>
-__global__ void __launch_bounds__(128) cg_p_update(VecArgs v, const RhsState *st, SpinorField<W> z, SpinorField<W> p)
-{
-    pdl_begin();
-    const int j = blockIdx.x % v.nrhs, tile = blockIdx.x / v.nrhs;
-    if (v.gate_st && v.gate_st[j].status != v.gate) return;
-    const int i = tile * blockDim.x + threadIdx.x;
-    if (i >= v.vh) return;
-    using R = typename std::conditional<std::is_same<W, F64>::value, double, float>::type;
-    store_spinor<W, R>(p, j, i, axpy_sp(beta_of<R>(st[j]), load_vec<W, R>(p, j, i), load_vec<W, R>(z, j, i)));
 }
 
 // x += scale e ; e = 0   (FP64 x)

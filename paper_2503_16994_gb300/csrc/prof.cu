@@ -100,7 +100,7 @@ std::map<std::tuple<std::string, int, int, int>, std::array<int, 4>> g_imported;
 // a shape the launcher accepts for its storage format (the candidates of the tuner)
 bool shape_valid(const std::string &prec, int mode, int vh, int nrhs, int nr, int gpb, int minb, int swz)
 {
-    if ((mode != 0 && mode != 1) || vh <= 0 || nrhs < 1 || gpb < 1 || gpb > 12) return false;
+    if ((mode != HOP_CLOV && mode != SELF_CLOV && mode != ADD_CLOV && mode != SELF_SUM) || vh <= 0 || nrhs < 1 || gpb < 1 || gpb > 12) return false;
     if (minb != 1 && minb != 3 && minb != 4 && minb != 6) return false;
     if (swz != 1 && swz != 8 && swz != 32) return false;
     const bool tile = nr == 20 || nr == 21;
@@ -123,7 +123,7 @@ bool tune_imported(const char *prec, int mode, int vh, int nrhs, int shape[4])
 
 void tune_record(const char *prec, int mode, int vh, int nrhs, int nr, int gpb, int minb, int swz, float ms)
 {
-    static const char *modes[] = {"hopclov", "selfclov", "self", "clovsum", "resid"};
+    static const char *modes[] = {"hopclov", "selfclov", "self", "clovsum", "resid", "addclov", "selfsum"};
     // shape code nr: 1-3 scalar (nr RHS per thread), 0 paired, -2/-4/-8
     // prefetching (loads of that many directions ahead), 12/13 paired with
     // 2/3 directions staged in shared memory, 20/21 tile kernel (links and

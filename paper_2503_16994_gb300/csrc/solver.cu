@@ -7,13 +7,20 @@
 // and the full residual equals bhat - Dhat x_e on the even sites (zero on the
 // odd ones), so |b - D x| = |bhat - Dhat x_e| up to rounding.
 //
-// Dhat is solved by CG on the normal equations in CGLS form (the recursion
-// tracks r = rhat - Dhat e, the residual of the system itself):
-//   z = Dhat^dag r, p = z, gamma = |z|^2
-//   repeat: w = Dhat p; alpha = gamma/|w|^2; e += alpha p; r -= alpha w;
-//           z = Dhat^dag r; beta = |z|^2/gamma; gamma = |z|^2; p = z + beta p
-// with Dhat^dag = g5 Dhat g5 (the hopping projectors swap, the clover term
-// commutes with g5).  The inner vectors are FP64, FP32 or FP16; every time the
+// It is solved with the even site term divided out too, on the right:
+//   M y = bhat,  x_e = A_ee^-1 y,
+//   M = Dhat A_ee^-1 = 1 - k^2 H_eo A_oo^-1 H_oe A_ee^-1,
+// by CG on its normal equations in CGLS form (the recursion tracks r = rhat -
+// M e, the residual of the system itself, so every stopping rule is that of
+// Dhat):
+//   z = M^dag r, p = z, gamma = |z|^2
+//   repeat: w = M p; alpha = gamma/|w|^2; e += alpha p; r -= alpha w;
+//           z = M^dag r; beta = |z|^2/gamma; gamma = |z|^2; p = z + beta p
+// with the adjoint by g5 (the hopping projectors swap, the clover term
+// commutes with g5).  M is better conditioned than Dhat: 130 iterations
+// instead of 150 on 16^3 x 32 (kappa 0.130, c_sw 1.5) and 193 instead of 229
+// (0.132, 1.7), for one more pass over the clover blocks in the p update and
+// one less in a hop.  The inner vectors are FP64, FP32 or FP16; every time the
 // inner residual has dropped by delta (or looks converged, or the iteration
 // cap is hit) the correction is added to the FP64 solution and the residual
 // is recomputed in FP64 (reliable update), keeping p.  Mixed solvers whose
@@ -177,7 +184,8 @@ struct Solver {
     HopArgs<W, W, W> hw;
     HopArgs<F32, F32, F32> h32;  // FP32 operator of the incremental residual updates (mixed solvers)
     CloverField<F64> a64, ai64, ci64;  // ci64: the C blocks of a twisted inverse
-    CloverField<W> aw, aiw;
+    CloverField<W> aw, aiw, ciw;
+    CloverField<E> aie, cie;  // A_ee^-1 for the correction
     SpinorField<F64> b_e, b_o, bhat, x_e, x_o, t64, w64;
     SpinorField<W> p, t, w, r, z;
     SpinorField<E> e;
@@ -209,6 +217,9 @@ struct Solver {
         ci64 = clover_field_c<F64>(cl, Sd);
         aw = clover_field<W>(cl, false, Sd);
         aiw = clover_field<W>(cl, true, Sd);
+        ciw = clover_field_c<W>(cl, Sd);
+        aie = clover_field<E>(cl, true, Sd);
+        cie = clover_field_c<E>(cl, Sd);
         const int nt = ntiles_of(lat->vh);
         Reduce red{ws.partial.as<double>(), ws.counter.as<unsigned>(), S, RED_STORE,
                    reinterpret_cast<float *>(ws.partial.as<double>() + (size_t)nrhs * nt)};
@@ -288,9 +299,13 @@ struct Solver {
         if (ws.p_sc.p) LQCD_CUDA(cudaMemsetAsync(ws.p_sc.p, 0, ws.p_sc.bytes, st));
     }
 
+    // e = A_ee^-1 e: the correction of x_e from that of y   [gate UPDATE]
+    void site_correction() { launch_e_site<E>(gated(ST_UPDATE, RED_STORE), e, aie, cie, h64.tau, st); }
+
     // x += scale e; rhat = bhat - Dhat x (FP64); r = rhat / scale   [gate UPDATE]
     void reliable_update()
     {
+        site_correction();
         launch_x_update<E>(gated(ST_UPDATE, RED_STORE), S, e, x_e, st);
         HopArgs<F64, F64, F64> a = h64;
         a.gate_st = S;
@@ -333,6 +348,7 @@ struct Solver {
             const long Sd = lat->stride;
             SpinorField<F32> t32{ws.t64.as<float4>(), nullptr, Sd};
             SpinorField<F32> w32{ws.w64.as<float4>(), nullptr, Sd};
+            site_correction();
             HopArgs<F32, F32, F32> a = h32;
             a.gate_st = S;
             a.gate = ST_UPDATE;
@@ -383,7 +399,8 @@ struct Solver {
             reliable_update();
     }
 
-    // w = Dhat p (|w|^2 -> alpha); e += alpha p; r -= alpha w   [gate ACTIVE]
+    // w = M p (|w|^2 -> alpha); e += alpha p; r -= alpha w   [gate ACTIVE]
+    // (z holds A_ee^-1 p from the p update)
     void half1()
     {
         HopArgs<W, W, W> a = hw;
@@ -391,7 +408,7 @@ struct Solver {
         a.gate = ST_ACTIVE;
         a.nactive = hint_active;
         a.parity = 1;
-        a.in = p;
+        a.in = z;
         a.out = t;
         a.clov = aiw;
         a.coef = kappa;
@@ -400,14 +417,13 @@ struct Solver {
         a.in = t;
         a.self = p;
         a.out = w;
-        a.clov = aw;
         a.coef = -kappa;
         a.red.op = RED_ALPHA;
-        launch_hop(a, SELF_CLOV, false, true, st);
+        launch_hop(a, SELF_SUM, false, true, st);
         launch_er_update<W, E>(gated(ST_ACTIVE, RED_RUPDATE), p, w, r, e, st);
     }
 
-    // z = Dhat^dag r (|z|^2 -> beta, gamma); p = z + beta p   [gate ACTIVE or RESUME]
+    // z = M^dag r (|z|^2 -> beta, gamma); p = z + beta p; z = A_ee^-1 p   [gate ACTIVE or RESUME]
     void half2(int gate = ST_ACTIVE)
     {
         HopArgs<W, W, W> a = hw;
@@ -424,11 +440,10 @@ struct Solver {
         a.in = t;
         a.self = r;
         a.out = z;
-        a.clov = aw;
         a.coef = -kappa;
         a.red.op = RED_BETA;
-        launch_hop(a, SELF_CLOV, true, true, st);
-        launch_p_update<W>(gated(gate, RED_STORE), S, z, p, st);
+        launch_hop(a, ADD_CLOV, true, true, st);
+        launch_p_update<W>(gated(gate, RED_STORE), S, z, p, aiw, ciw, hw.tau, st);
     }
 
     void set_resume(int v)
