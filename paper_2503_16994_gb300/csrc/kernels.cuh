@@ -12,7 +12,13 @@ namespace lqcd {
 // ---------------------------------------------------------------------------
 // ST_RESUME: just updated in FP64 while the others went on (batched
 // solves); runs the second half of its iteration, then becomes ST_ACTIVE.
-enum RhsStatus : int { ST_DONE = 0, ST_ACTIVE = 1, ST_UPDATE = 2, ST_MAXITER = 3, ST_IDLE = 4, ST_RESUME = 5 };
+// ST_FINAL: the recursion's residual has reached the target; the correction is
+// added and the FP64 residual of the full lattice that ends every solve
+// decides (after a miss the next ones are checked like any update).
+enum RhsStatus : int {
+    ST_DONE = 0, ST_ACTIVE = 1, ST_UPDATE = 2, ST_MAXITER = 3, ST_IDLE = 4, ST_RESUME = 5, ST_FINAL = 6
+};
+enum RhsTrust : int { TRUST_NONE = 0, TRUST_OPEN = 1, TRUST_USED = 2 };
 
 struct RhsState {
     double gamma;    // |z|^2, z = Dhat^dag r (CGLS)
@@ -30,6 +36,7 @@ struct RhsState {
     int updates;
     int maxiter;
     int resume;      // status after an FP64 residual that did not finish: ST_ACTIVE or ST_RESUME
+    int trust;       // TRUST_OPEN: a converged recursion goes to ST_FINAL instead of ST_UPDATE
     float alpha_f, beta_f;  // alpha, beta in FP32 (the FP16/FP32 vector kernels; converted once)
 };
 
@@ -70,12 +77,18 @@ __device__ __forceinline__ void apply_op(const Reduce &r, int j, double sum)
     case RED_RUPDATE:
         s.rr = sum;
         s.iter += 1;
-        if (sum <= s.delta2 * s.rr_ref || s.scale * s.scale * sum <= s.target2 || s.iter >= s.maxiter ||
-            !(sum == sum))
+        if (s.trust == TRUST_OPEN && s.scale * s.scale * sum <= s.target2) {
+            s.status = ST_FINAL;
+            s.trust = TRUST_USED;
+        } else if (sum <= s.delta2 * s.rr_ref || s.scale * s.scale * sum <= s.target2 || s.iter >= s.maxiter ||
+                   !(sum == sum)) {
             s.status = ST_UPDATE;
+        }
         break;
     case RED_RHAT:
         s.updates += 1;
+        // far above the recursion's residual: what it gathered is of no use, begin again (beta = 0)
+        if (sum > 4.0 * s.scale * s.scale * s.rr) s.gamma = 0.0;
         s.rr = sum / (s.scale * s.scale);
         s.rr_ref = s.rr;
         s.anchor2 = sum;
