@@ -12,6 +12,7 @@
 namespace lqcd {
 
 constexpr int kStageWords = 8;  // 16-byte words per direction and thread
+constexpr int kStageThreads = 128;  // threads per block (kBlock)
 
 __device__ __forceinline__ void cp_async16(unsigned dst, const void *src)
 {
@@ -69,22 +70,23 @@ __device__ __forceinline__ void stage_issue(const FastHop<F16> &a, int ja, int j
 {
     constexpr int MU = D / 2, DIR = (D & 1) ? -1 : 1;
     const long st = a.in.stride;
-    const uint4 *pa = a.in.p + (long)ja * 3 * st + y;
-    const uint4 *pb = a.in.p + (long)jb * 3 * st + y;
+    const uint4 *pa = a.in.p + (long)ja * 3 * st;
+    const uint4 *pb = a.in.p + (long)jb * 3 * st;
     const int par = DIR > 0 ? a.parity : (a.parity ^ 1);
-    const long lq = (long)(par * 4 + MU) * a.U.stride + (DIR > 0 ? i : y);
-    const unsigned ws = blockDim.x * 16u;
-    const unsigned d = unsigned(__cvta_generic_to_shared(stage + slot * kStageWords * blockDim.x + threadIdx.x));
-    cp_async16(d, pa);
-    cp_async16(d + ws, pa + st);
-    cp_async16(d + 2 * ws, pa + 2 * st);
-    cp_async16(d + 3 * ws, pb);
-    cp_async16(d + 4 * ws, pb + st);
-    cp_async16(d + 5 * ws, pb + 2 * st);
-    cp_async16(d + 6 * ws, a.U.p + lq);
-    cp_async8(d + 7 * ws, a.U.p2 + lq);
-    cp_async4(d + 7 * ws + 8, a.in.scale + (long)ja * st + y);
-    cp_async4(d + 7 * ws + 12, a.in.scale + (long)jb * st + y);
+    const long lq = (long)(par * 4 + MU) * a.U.stride;
+    const int l = DIR > 0 ? i : y;
+    constexpr unsigned ws = kStageThreads * 16u;
+    const unsigned d = unsigned(__cvta_generic_to_shared(stage + slot * kStageWords * kStageThreads + threadIdx.x));
+    cp_async16(d, at(pa, y));
+    cp_async16(d + ws, at(pa + st, y));
+    cp_async16(d + 2 * ws, at(pa + 2 * st, y));
+    cp_async16(d + 3 * ws, at(pb, y));
+    cp_async16(d + 4 * ws, at(pb + st, y));
+    cp_async16(d + 5 * ws, at(pb + 2 * st, y));
+    cp_async16(d + 6 * ws, at(a.U.p + lq, l));
+    cp_async8(d + 7 * ws, at(a.U.p2 + lq, l));
+    cp_async4(d + 7 * ws + 8, at(a.in.scale + (long)ja * st, y));
+    cp_async4(d + 7 * ws + 12, at(a.in.scale + (long)jb * st, y));
     cp_async_commit();
 }
 
@@ -94,7 +96,7 @@ __device__ __forceinline__ void stage_compute(const FastHop<F16> &a, const uint4
 {
     constexpr int MU = D / 2, DIR = (D & 1) ? -1 : 1;
     constexpr int SP = DIR > 0 ? -SG : SG;
-    const int nt = blockDim.x;
+    constexpr int nt = kStageThreads;
     const uint4 *s0 = stage + slot * kStageWords * nt + threadIdx.x;
     uint4 w[kStageWords];
 #pragma unroll
