@@ -45,21 +45,24 @@ __device__ __forceinline__ void site_inverse(const CloverField<C> &cl, const Clo
     }
 }
 
-// p = z + beta p; z = A_ee^-1 p, the input of the next application of the
-// operator.  Bound by memory (z, p in and out and the clover block, which the
-// right-hand sides of a site share in cache): 152 us for 12 right-hand sides on
-// 24^3 x 48, 5.7 TB/s (170 us with the clover words loaded after the vectors;
-// without z = A_ee^-1 p it was 87 us, for 380 iterations instead of 314).
-template <class W>
+// e += alpha p; p = z + beta p; z = A_ee^-1 p, the input of the next application
+// of the operator.  e is updated here, where p is read anyway, and not with r
+// (cg_r_update).  Bound by memory (p, z and e in and out and the clover block,
+// which the right-hand sides of a site share in cache): for 12 right-hand sides
+// on 24^3 x 48 in FP16 240 us, 6.8 TB/s, and 108 for r, where p and z took 152 us
+// (5.7 TB/s) and r with e 239; one right-hand side on 32^3 x 64 82 + 51 us,
+// before 53 + 92.  (The clover words loaded after the vectors cost 18 us more.)
+template <class W, class E>
 __global__ void __launch_bounds__(128) cg_p_update(VecArgs v, const RhsState *st, SpinorField<W> z, SpinorField<W> p,
-                                                   CloverField<W> cl, CloverField<W> cl2, double tau)
+                                                   SpinorField<E> e, CloverField<W> cl, CloverField<W> cl2,
+                                                   double tau)
 {
     const int j = blockIdx.x % v.nrhs, tile = blockIdx.x / v.nrhs;
     if (v.gate_st && v.gate_st[j].status != v.gate) return;
     const int i = tile * blockDim.x + threadIdx.x;
     if (i >= v.vh) return;
     using R = typename real_of<W>::type;
-    const R be = st[j].beta_f;
+    const R al = alpha_of<R>(st[j]), be = st[j].beta_f;
     R x[24], y[24];
     // FP16: the clover words are on their way with the vectors (36 registers)
     uint4 cw[W::W == 8 ? 9 : 1];
@@ -68,6 +71,10 @@ __global__ void __launch_bounds__(128) cg_p_update(VecArgs v, const RhsState *st
         for (int k = 0; k < 9; ++k) cw[k] = __ldg(cl.p + k * cl.stride + i);
     }
     load_scaled<W, R>(p, j, i, x);
+    load_scaled<E, R>(e, j, i, y);
+#pragma unroll
+    for (int q = 0; q < 24; ++q) y[q] = fma(al, x[q], y[q]);
+    store_raw<E, R>(e, j, i, y);
     load_scaled<W, R>(z, j, i, y);
 #pragma unroll
     for (int q = 0; q < 24; ++q) x[q] = fma(be, x[q], y[q]);
@@ -98,19 +105,21 @@ __global__ void __launch_bounds__(128) cg_p_update(VecArgs v, const RhsState *st
 // the site blocks are 264 FP64 instructions, and on a small lattice a block of
 // 128 sites with all of them kept one SM busy for 8 us.
 __global__ void __launch_bounds__(32) cg_p_update64(VecArgs v, const RhsState *st, SpinorField<F64> z,
-                                                    SpinorField<F64> p, CloverField<F64> cl, CloverField<F64> cl2,
-                                                    double tau)
+                                                    SpinorField<F64> p, SpinorField<F64> e, CloverField<F64> cl,
+                                                    CloverField<F64> cl2, double tau)
 {
     pdl_begin();
     const int blk = blockIdx.y, j = blockIdx.x % v.nrhs, i = (blockIdx.x / v.nrhs) * 32 + threadIdx.x;
     if (v.gate_st && v.gate_st[j].status != v.gate) return;
     if (i >= v.vh) return;
-    const double be = st[j].beta;
+    const double al = st[j].alpha, be = st[j].beta;
+    double2 *eb = e.p + ((long)j * 12 + 6 * blk) * e.stride + i;
     double2 *pb = p.p + ((long)j * 12 + 6 * blk) * p.stride + i, *zb = z.p + ((long)j * 12 + 6 * blk) * z.stride + i;
     double x[12], y[12], A[36];
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-        const double2 a = pb[k * p.stride], b = zb[k * z.stride];
+        const double2 a = pb[k * p.stride], b = zb[k * z.stride], c = eb[k * e.stride];
+        eb[k * e.stride] = make_double2(fma(al, a.x, c.x), fma(al, a.y, c.y));
         x[2 * k] = fma(be, a.x, b.x);
         x[2 * k + 1] = fma(be, a.y, b.y);
         pb[k * p.stride] = make_double2(x[2 * k], x[2 * k + 1]);
@@ -127,10 +136,11 @@ __global__ void __launch_bounds__(32) cg_p_update64(VecArgs v, const RhsState *s
     for (int k = 0; k < 6; ++k) zb[k * z.stride] = make_double2(y[2 * k], y[2 * k + 1]);
 }
 
-// e = A_ee^-1 e, the correction in terms of the solution (residual updates)
-template <class E>
-__global__ void __launch_bounds__(128) cg_e_site(VecArgs v, SpinorField<E> e, CloverField<E> cl, CloverField<E> cl2,
-                                                 double tau)
+// e = A_ee^-1 (e + alpha p), the correction in terms of the solution, with the
+// step that cg_p_update would have added next (residual updates)
+template <class W, class E>
+__global__ void __launch_bounds__(128) cg_e_site(VecArgs v, const RhsState *st, SpinorField<W> p, SpinorField<E> e,
+                                                 CloverField<E> cl, CloverField<E> cl2, double tau)
 {
     const int j = blockIdx.x % v.nrhs, tile = blockIdx.x / v.nrhs;
     if (v.gate_st && v.gate_st[j].status != v.gate) return;
@@ -139,6 +149,10 @@ __global__ void __launch_bounds__(128) cg_e_site(VecArgs v, SpinorField<E> e, Cl
     using R = typename real_of<E>::type;
     R x[24], y[24];
     load_scaled<E, R>(e, j, i, x);
+    load_scaled<W, R>(p, j, i, y);
+    const R al = alpha_of<R>(st[j]);
+#pragma unroll
+    for (int q = 0; q < 24; ++q) x[q] = fma(al, y[q], x[q]);
     site_inverse<E, R>(cl, cl2, R(tau), i, x, y);
     store_raw<E, R>(e, j, i, y);
 }
@@ -204,42 +218,42 @@ static unsigned grid_of(const VecArgs &v) { return unsigned(v.ntiles * v.nrhs); 
 // right-hand sides a launch is expected to work on (accounting only)
 static double nact(const VecArgs &v) { return v.nactive >= 0 ? std::min(v.nactive, v.nrhs) : v.nrhs; }
 
-template <class W, class E>
-void launch_er_update(const VecArgs &v, SpinorField<W> p, SpinorField<W> w, SpinorField<W> r, SpinorField<E> e,
-                      cudaStream_t st)
+template <class W>
+void launch_r_update(const VecArgs &v, SpinorField<W> w, SpinorField<W> r, cudaStream_t st)
 {
-    ProfScope prof(prec_name<W>() == std::string("f64") ? "cg_er_update_f64" : (prec_name<W>() == std::string("f32") ? "cg_er_update_f32" : "cg_er_update_f16"),
-                   double(v.vh) * nact(v) * (4.0 * spinor_bytes<W>() + 2.0 * spinor_bytes<E>()), st);
+    ProfScope prof("cg_r_update", double(v.vh) * nact(v) * 3.0 * spinor_bytes<W>(), st);
     if constexpr (std::is_same<W, F64>::value)
-        launch_pdl(cg_er_update<W, E>, dim3(grid_of(v)), kBlock, 0, st, v, p, w, r, e);
+        launch_pdl(cg_r_update<W>, dim3(grid_of(v)), kBlock, 0, st, v, w, r);
     else
-        cg_er_update<W, E><<<grid_of(v), kBlock, 0, st>>>(v, p, w, r, e);
+        cg_r_update<W><<<grid_of(v), kBlock, 0, st>>>(v, w, r);
     LQCD_CHECK_LAUNCH();
 }
 
-template <class W>
-void launch_p_update(const VecArgs &v, const RhsState *s, SpinorField<W> z, SpinorField<W> p, CloverField<W> cl,
-                     CloverField<W> cl2, double tau, cudaStream_t st)
+template <class W, class E>
+void launch_p_update(const VecArgs &v, const RhsState *s, SpinorField<W> z, SpinorField<W> p, SpinorField<E> e,
+                     CloverField<W> cl, CloverField<W> cl2, double tau, cudaStream_t st)
 {
     ProfScope prof("cg_p_update",
-                   double(v.vh) * (nact(v) * 4.0 * spinor_bytes<W>() + (tau != 0.0 ? 2.0 : 1.0) * clover_bytes<W>()),
+                   double(v.vh) * (nact(v) * (4.0 * spinor_bytes<W>() + 2.0 * spinor_bytes<E>()) +
+                                   (tau != 0.0 ? 2.0 : 1.0) * clover_bytes<W>()),
                    st);
     if constexpr (std::is_same<W, F64>::value)
-        launch_pdl(cg_p_update64, dim3(unsigned((v.vh + 31) / 32) * unsigned(v.nrhs), 2), 32, 0, st, v, s, z, p, cl,
-                   cl2, tau);
+        launch_pdl(cg_p_update64, dim3(unsigned((v.vh + 31) / 32) * unsigned(v.nrhs), 2), 32, 0, st, v, s, z, p, e,
+                   cl, cl2, tau);
     else
-        cg_p_update<W><<<grid_of(v), kBlock, 0, st>>>(v, s, z, p, cl, cl2, tau);
+        cg_p_update<W, E><<<grid_of(v), kBlock, 0, st>>>(v, s, z, p, e, cl, cl2, tau);
     LQCD_CHECK_LAUNCH();
 }
 
-template <class E>
-void launch_e_site(const VecArgs &v, SpinorField<E> e, CloverField<E> cl, CloverField<E> cl2, double tau,
-                   cudaStream_t st)
+template <class W, class E>
+void launch_e_site(const VecArgs &v, const RhsState *s, SpinorField<W> p, SpinorField<E> e, CloverField<E> cl,
+                   CloverField<E> cl2, double tau, cudaStream_t st)
 {
     ProfScope prof("cg_e_site",
-                   double(v.vh) * (nact(v) * 2.0 * spinor_bytes<E>() + (tau != 0.0 ? 2.0 : 1.0) * clover_bytes<E>()),
+                   double(v.vh) * (nact(v) * (2.0 * spinor_bytes<E>() + spinor_bytes<W>()) +
+                                   (tau != 0.0 ? 2.0 : 1.0) * clover_bytes<E>()),
                    st);
-    cg_e_site<E><<<grid_of(v), kBlock, 0, st>>>(v, e, cl, cl2, tau);
+    cg_e_site<W, E><<<grid_of(v), kBlock, 0, st>>>(v, s, p, e, cl, cl2, tau);
     LQCD_CHECK_LAUNCH();
 }
 
@@ -293,22 +307,21 @@ template void launch_convert<F64, F32>(long, int, SpinorField<F64>, SpinorField<
 template void launch_convert<F64, F16>(long, int, SpinorField<F64>, SpinorField<F16>, cudaStream_t);
 template void launch_convert<F32, F64>(long, int, SpinorField<F32>, SpinorField<F64>, cudaStream_t);
 template void launch_convert<F16, F64>(long, int, SpinorField<F16>, SpinorField<F64>, cudaStream_t);
-template void launch_er_update<F64, F64>(const VecArgs &, SpinorField<F64>, SpinorField<F64>, SpinorField<F64>,
-                                         SpinorField<F64>, cudaStream_t);
-template void launch_er_update<F32, F32>(const VecArgs &, SpinorField<F32>, SpinorField<F32>, SpinorField<F32>,
-                                         SpinorField<F32>, cudaStream_t);
-template void launch_er_update<F16, F32>(const VecArgs &, SpinorField<F16>, SpinorField<F16>, SpinorField<F16>,
-                                         SpinorField<F32>, cudaStream_t);
-template void launch_p_update<F64>(const VecArgs &, const RhsState *, SpinorField<F64>, SpinorField<F64>, CloverField<F64>,
-                                   CloverField<F64>, double, cudaStream_t);
-template void launch_p_update<F32>(const VecArgs &, const RhsState *, SpinorField<F32>, SpinorField<F32>, CloverField<F32>,
-                                   CloverField<F32>, double, cudaStream_t);
-template void launch_p_update<F16>(const VecArgs &, const RhsState *, SpinorField<F16>, SpinorField<F16>, CloverField<F16>,
-                                   CloverField<F16>, double, cudaStream_t);
-template void launch_e_site<F64>(const VecArgs &, SpinorField<F64>, CloverField<F64>, CloverField<F64>, double,
-                                 cudaStream_t);
-template void launch_e_site<F32>(const VecArgs &, SpinorField<F32>, CloverField<F32>, CloverField<F32>, double,
-                                 cudaStream_t);
+template void launch_r_update<F64>(const VecArgs &, SpinorField<F64>, SpinorField<F64>, cudaStream_t);
+template void launch_r_update<F32>(const VecArgs &, SpinorField<F32>, SpinorField<F32>, cudaStream_t);
+template void launch_r_update<F16>(const VecArgs &, SpinorField<F16>, SpinorField<F16>, cudaStream_t);
+template void launch_p_update<F64, F64>(const VecArgs &, const RhsState *, SpinorField<F64>, SpinorField<F64>,
+                                        SpinorField<F64>, CloverField<F64>, CloverField<F64>, double, cudaStream_t);
+template void launch_p_update<F32, F32>(const VecArgs &, const RhsState *, SpinorField<F32>, SpinorField<F32>,
+                                        SpinorField<F32>, CloverField<F32>, CloverField<F32>, double, cudaStream_t);
+template void launch_p_update<F16, F32>(const VecArgs &, const RhsState *, SpinorField<F16>, SpinorField<F16>,
+                                        SpinorField<F32>, CloverField<F16>, CloverField<F16>, double, cudaStream_t);
+template void launch_e_site<F64, F64>(const VecArgs &, const RhsState *, SpinorField<F64>, SpinorField<F64>,
+                                      CloverField<F64>, CloverField<F64>, double, cudaStream_t);
+template void launch_e_site<F32, F32>(const VecArgs &, const RhsState *, SpinorField<F32>, SpinorField<F32>,
+                                      CloverField<F32>, CloverField<F32>, double, cudaStream_t);
+template void launch_e_site<F16, F32>(const VecArgs &, const RhsState *, SpinorField<F16>, SpinorField<F32>,
+                                      CloverField<F32>, CloverField<F32>, double, cudaStream_t);
 template void launch_x_update<F64>(const VecArgs &, const RhsState *, SpinorField<F64>, SpinorField<F64>, cudaStream_t);
 template void launch_x_update<F32>(const VecArgs &, const RhsState *, SpinorField<F32>, SpinorField<F64>, cudaStream_t);
 template void launch_r_replace<F64, F64>(const VecArgs &, SpinorField<F64>, SpinorField<F64>, SpinorField<F64>,

@@ -89,6 +89,7 @@ __device__ __forceinline__ void apply_op(const Reduce &r, int j, double sum)
         s.updates += 1;
         // far above the recursion's residual: what it gathered is of no use, begin again (beta = 0)
         if (sum > 4.0 * s.scale * s.scale * s.rr) s.gamma = 0.0;
+        s.alpha = s.alpha_f = 0.f;  // alpha p is in e (cg_e_site), and e in x
         s.rr = sum / (s.scale * s.scale);
         s.rr_ref = s.rr;
         s.anchor2 = sum;
@@ -100,6 +101,7 @@ __device__ __forceinline__ void apply_op(const Reduce &r, int j, double sum)
             s.status = s.resume;
         break;
     case RED_RHAT_COARSE:
+        s.alpha = s.alpha_f = 0.f;
         s.rr = sum / (s.scale * s.scale);
         s.rr_ref = s.rr;
         s.status = (sum == sum) ? s.resume : ST_UPDATE;  // a NaN goes to the FP64 update
@@ -324,15 +326,15 @@ __device__ __forceinline__ spinor<R> load_vec(const SpinorField<S> &f, int j, in
     else return load_spinor<S, R>(f, j, i);
 }
 
-// e += alpha p ; r -= alpha w ; |r|^2 -> RED_RUPDATE
 template <typename R> __device__ __forceinline__ R alpha_of(const RhsState &s)
 {
     if constexpr (std::is_same<R, float>::value) return s.alpha_f;
     else return s.alpha;
 }
-template <class W, class E>
-__global__ void __launch_bounds__(128) cg_er_update(VecArgs v, SpinorField<W> p, SpinorField<W> w, SpinorField<W> r,
-                                                    SpinorField<E> e)
+
+// r -= alpha w ; |r|^2 -> RED_RUPDATE  (e += alpha p follows where p is read next: cg_p_update, cg_e_site)
+template <class W>
+__global__ void __launch_bounds__(128) cg_r_update(VecArgs v, SpinorField<W> w, SpinorField<W> r)
 {
     pdl_begin();
     const int j = blockIdx.x % v.nrhs, tile = blockIdx.x / v.nrhs;
@@ -340,11 +342,9 @@ __global__ void __launch_bounds__(128) cg_er_update(VecArgs v, SpinorField<W> p,
     const int i = tile * blockDim.x + threadIdx.x;
     double n2 = 0.0;
     if (i < v.vh) {
-        using R = typename std::conditional<std::is_same<E, F64>::value, double, float>::type;
+        using R = typename std::conditional<std::is_same<W, F64>::value, double, float>::type;
         const R al = alpha_of<R>(v.red.st[j]);
-        const spinor<R> pv = load_vec<W, R>(p, j, i), ev = load_vec<E, R>(e, j, i);
         const spinor<R> wv = load_vec<W, R>(w, j, i), rv = load_vec<W, R>(r, j, i);
-        store_spinor<E, R>(e, j, i, axpy_sp(al, pv, ev));
         n2 = store_spinor<W, R>(r, j, i, axpy_sp(-al, wv, rv));
     }
     reduce_finish(v.red, j, tile, v.ntiles, n2);

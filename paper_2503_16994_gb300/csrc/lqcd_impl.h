@@ -279,16 +279,15 @@ void launch_hop(const HopArgs<S, L, C> &a, int mode, bool dag, bool norm, cudaSt
 void launch_dirac(const HopArgs<F64, F64, F64> &a, const double *in, double *out, bool dag, cudaStream_t st);
 
 // vector kernels (blas_*.cu)
-template <class W, class E>
-void launch_er_update(const VecArgs &v, SpinorField<W> p, SpinorField<W> w, SpinorField<W> r, SpinorField<E> e,
-                      cudaStream_t st);
 template <class W>
-void launch_p_update(const VecArgs &v, const RhsState *s, SpinorField<W> z, SpinorField<W> p, CloverField<W> cl,
-                     CloverField<W> cl2, double tau, cudaStream_t st);
-// e = A_ee^-1 e
-template <class E>
-void launch_e_site(const VecArgs &v, SpinorField<E> e, CloverField<E> cl, CloverField<E> cl2, double tau,
-                   cudaStream_t st);
+void launch_r_update(const VecArgs &v, SpinorField<W> w, SpinorField<W> r, cudaStream_t st);
+template <class W, class E>
+void launch_p_update(const VecArgs &v, const RhsState *s, SpinorField<W> z, SpinorField<W> p, SpinorField<E> e,
+                     CloverField<W> cl, CloverField<W> cl2, double tau, cudaStream_t st);
+// e = A_ee^-1 (e + alpha p)
+template <class W, class E>
+void launch_e_site(const VecArgs &v, const RhsState *s, SpinorField<W> p, SpinorField<E> e, CloverField<E> cl,
+                   CloverField<E> cl2, double tau, cudaStream_t st);
 template <class E>
 void launch_x_update(const VecArgs &v, const RhsState *s, SpinorField<E> e, SpinorField<F64> x, cudaStream_t st);
 template <class W, class WI>

@@ -172,7 +172,10 @@ __global__ void set_resume_kernel(RhsState *s, int nrhs, int v)
 __global__ void status_change_kernel(RhsState *s, int nrhs, int from, int to)
 {
     int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < nrhs && s[j].status == from) s[j].status = to;
+    if (j < nrhs && s[j].status == from) {
+        s[j].status = to;
+        s[j].alpha = s[j].alpha_f = 0.f;  // alpha p is in e (cg_e_site)
+    }
 }
 
 template <class W, class E>
@@ -302,8 +305,11 @@ struct Solver {
         if (ws.p_sc.p) LQCD_CUDA(cudaMemsetAsync(ws.p_sc.p, 0, ws.p_sc.bytes, st));
     }
 
-    // e = A_ee^-1 e: the correction of x_e from that of y   [gate UPDATE]
-    void site_correction() { launch_e_site<E>(gated(ST_UPDATE, RED_STORE), e, aie, cie, h64.tau, st); }
+    // e = A_ee^-1 (e + alpha p): the correction of x_e from that of y   [gate]
+    void site_correction(int gate = ST_UPDATE)
+    {
+        launch_e_site<W, E>(gated(gate, RED_STORE), S, p, e, aie, cie, h64.tau, st);
+    }
 
     // x += scale e; rhat = bhat - Dhat x (FP64); r = rhat / scale   [gate UPDATE]
     void reliable_update()
@@ -401,7 +407,7 @@ struct Solver {
     void update_best()
     {
         if (any_status(ST_FINAL)) {
-            launch_e_site<E>(gated(ST_FINAL, RED_STORE), e, aie, cie, h64.tau, st);
+            site_correction(ST_FINAL);
             launch_x_update<E>(gated(ST_FINAL, RED_STORE), S, e, x_e, st);
             status_change_kernel<<<(nrhs + 31) / 32, 32, 0, st>>>(S, nrhs, ST_FINAL, ST_DONE);
             LQCD_CHECK_LAUNCH();
@@ -413,7 +419,7 @@ struct Solver {
             reliable_update();
     }
 
-    // w = M p (|w|^2 -> alpha); e += alpha p; r -= alpha w   [gate ACTIVE]
+    // w = M p (|w|^2 -> alpha); r -= alpha w   [gate ACTIVE]
     // (z holds A_ee^-1 p from the p update)
     void half1()
     {
@@ -434,10 +440,10 @@ struct Solver {
         a.coef = -kappa;
         a.red.op = RED_ALPHA;
         launch_hop(a, SELF_SUM, false, true, st);
-        launch_er_update<W, E>(gated(ST_ACTIVE, RED_RUPDATE), p, w, r, e, st);
+        launch_r_update<W>(gated(ST_ACTIVE, RED_RUPDATE), w, r, st);
     }
 
-    // z = M^dag r (|z|^2 -> beta, gamma); p = z + beta p; z = A_ee^-1 p   [gate ACTIVE or RESUME]
+    // z = M^dag r (|z|^2 -> beta, gamma); e += alpha p; p = z + beta p; z = A_ee^-1 p   [gate ACTIVE or RESUME]
     void half2(int gate = ST_ACTIVE)
     {
         HopArgs<W, W, W> a = hw;
@@ -457,7 +463,7 @@ struct Solver {
         a.coef = -kappa;
         a.red.op = RED_BETA;
         launch_hop(a, ADD_CLOV, true, true, st);
-        launch_p_update<W>(gated(gate, RED_STORE), S, z, p, aiw, ciw, hw.tau, st);
+        launch_p_update<W, E>(gated(gate, RED_STORE), S, z, p, e, aiw, ciw, hw.tau, st);
     }
 
     void set_resume(int v)
