@@ -49,8 +49,8 @@ __device__ __forceinline__ void site_inverse(const CloverField<C> &cl, const Clo
 // of the operator.  e is updated here, where p is read anyway, and not with r
 // (cg_r_update).  Bound by memory (p, z and e in and out and the clover block,
 // which the right-hand sides of a site share in cache): for 12 right-hand sides
-// on 24^3 x 48 in FP16 240 us, 6.8 TB/s, and 108 for r, where p and z took 152 us
-// (5.7 TB/s) and r with e 239; one right-hand side on 32^3 x 64 82 + 51 us,
+// on 24^3 x 48 in FP16 240 us, 6.8 TB/s, and 101 for r, where p and z took 152 us
+// (5.7 TB/s) and r with e 239; one right-hand side on 32^3 x 64 82 + 39 us,
 // before 53 + 92.  (The clover words loaded after the vectors cost 18 us more.)
 template <class W, class E>
 __global__ void __launch_bounds__(128) cg_p_update(VecArgs v, const RhsState *st, SpinorField<W> z, SpinorField<W> p,
@@ -214,6 +214,11 @@ void launch_partial_finish(const Reduce &r, int ntiles, int nrhs, const RhsState
     LQCD_CHECK_LAUNCH();
 }
 
+// From here cg_r_update takes four tiles per block: the chip holds about 1200 of
+// its blocks, so four times fewer still fill it.  In FP16 8192 tiles (one
+// right-hand side on 32^3 x 64) take 39 us instead of 51 and 31104 (12 on
+// 24^3 x 48) 101 instead of 108; fewer tiles than 4096 keep a block each.
+constexpr unsigned kManyTiles = 4096;
 static unsigned grid_of(const VecArgs &v) { return unsigned(v.ntiles * v.nrhs); }
 // right-hand sides a launch is expected to work on (accounting only)
 static double nact(const VecArgs &v) { return v.nactive >= 0 ? std::min(v.nactive, v.nrhs) : v.nrhs; }
@@ -222,10 +227,15 @@ template <class W>
 void launch_r_update(const VecArgs &v, SpinorField<W> w, SpinorField<W> r, cudaStream_t st)
 {
     ProfScope prof("cg_r_update", double(v.vh) * nact(v) * 3.0 * spinor_bytes<W>(), st);
-    if constexpr (std::is_same<W, F64>::value)
-        launch_pdl(cg_r_update<W>, dim3(grid_of(v)), kBlock, 0, st, v, w, r);
-    else
-        cg_r_update<W><<<grid_of(v), kBlock, 0, st>>>(v, w, r);
+    const bool many = grid_of(v) >= kManyTiles;
+    const unsigned grid = many ? unsigned((v.ntiles + 3) / 4) * unsigned(v.nrhs) : grid_of(v);
+    if constexpr (std::is_same<W, F64>::value) {
+        if (many) launch_pdl(cg_r_update<W, 4>, dim3(grid), kBlock, 0, st, v, w, r);
+        else launch_pdl(cg_r_update<W, 1>, dim3(grid), kBlock, 0, st, v, w, r);
+    } else {
+        if (many) cg_r_update<W, 4><<<grid, kBlock, 0, st>>>(v, w, r);
+        else cg_r_update<W, 1><<<grid, kBlock, 0, st>>>(v, w, r);
+    }
     LQCD_CHECK_LAUNCH();
 }
 

@@ -126,31 +126,50 @@ __device__ __forceinline__ double block_sum4(double v, double *sh)
     return warp_sum((t[0] + t[1]) + (t[2] + t[3]));
 }
 
-// Block-wide sum of v, written as this block's partial; the last block of
-// RHS j to arrive sums all partials in a fixed order (deterministic) and
-// applies the operation.  Must be called by every thread of the block (128).
-__device__ __forceinline__ void reduce_finish(const Reduce &r, int j, int tile, int ntiles, double v)
+// Block-wide sums of v[0..n), written as the partials of tiles tile .. tile +
+// n - 1; the last block of RHS j to arrive sums all partials in a fixed order
+// (deterministic, and the same for every n) and applies the operation.  Must be
+// called by every thread of the block (128).
+template <int K>
+__device__ __forceinline__ void reduce_finish(const Reduce &r, int j, int tile, int ntiles, const double (&v)[K])
 {
     __shared__ double sh[128];
     __shared__ int last;
-    double s = block_sum4(v, sh);
+    const int n = min(K, ntiles - tile);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const double s = block_sum4(v[k], sh);
+        if (threadIdx.x == 0 && k < n) r.partial[(long)j * ntiles + tile + k] = s;
+    }
     if (threadIdx.x == 0) {
-        r.partial[(long)j * ntiles + tile] = s;
         __threadfence();
-        unsigned prev = atomicAdd(&r.counter[j], 1u);
-        last = (prev == (unsigned)(ntiles - 1));
+        const unsigned prev = atomicAdd(&r.counter[j], unsigned(n));
+        last = prev + n == unsigned(ntiles);
     }
     __syncthreads();
     if (last) {
         __threadfence();
         double t = 0.0;
-        for (int k = threadIdx.x; k < ntiles; k += blockDim.x) t += __ldcg(r.partial + (long)j * ntiles + k);
+        const double *p = r.partial + (long)j * ntiles;
+        for (int k = threadIdx.x; k < ntiles; k += 8 * blockDim.x) {
+            double q[8];  // eight loads in flight
+#pragma unroll
+            for (int u = 0; u < 8; ++u) q[u] = k + u * blockDim.x < ntiles ? __ldcg(p + k + u * blockDim.x) : 0.0;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) t += q[u];
+        }
         t = block_sum4(t, sh);
         if (threadIdx.x == 0) {
             r.counter[j] = 0;
             apply_op(r, j, t);
         }
     }
+}
+
+__device__ __forceinline__ void reduce_finish(const Reduce &r, int j, int tile, int ntiles, double v)
+{
+    const double a[1] = {v};
+    reduce_finish<1>(r, j, tile, ntiles, a);
 }
 
 template <typename T>
@@ -332,22 +351,29 @@ template <typename R> __device__ __forceinline__ R alpha_of(const RhsState &s)
     else return s.alpha;
 }
 
-// r -= alpha w ; |r|^2 -> RED_RUPDATE  (e += alpha p follows where p is read next: cg_p_update, cg_e_site)
-template <class W>
+// r -= alpha w ; |r|^2 -> RED_RUPDATE  (e += alpha p follows where p is read
+// next: cg_p_update, cg_e_site).  K tiles per block: each block waits for its
+// stores (the fence before its partials count) and for an atomic, 1.7 of the 4 us
+// that a block of one tile lives.
+template <class W, int K>
 __global__ void __launch_bounds__(128) cg_r_update(VecArgs v, SpinorField<W> w, SpinorField<W> r)
 {
     pdl_begin();
-    const int j = blockIdx.x % v.nrhs, tile = blockIdx.x / v.nrhs;
+    const int j = blockIdx.x % v.nrhs, tile = blockIdx.x / v.nrhs * K;
     if (v.gate_st && v.gate_st[j].status != v.gate) return;
-    const int i = tile * blockDim.x + threadIdx.x;
-    double n2 = 0.0;
-    if (i < v.vh) {
-        using R = typename std::conditional<std::is_same<W, F64>::value, double, float>::type;
-        const R al = alpha_of<R>(v.red.st[j]);
-        const spinor<R> wv = load_vec<W, R>(w, j, i), rv = load_vec<W, R>(r, j, i);
-        n2 = store_spinor<W, R>(r, j, i, axpy_sp(-al, wv, rv));
+    using R = typename std::conditional<std::is_same<W, F64>::value, double, float>::type;
+    const R al = alpha_of<R>(v.red.st[j]);
+    double n2[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        n2[k] = 0.0;
+        const int i = (tile + k) * blockDim.x + threadIdx.x;
+        if (i < v.vh) {
+            const spinor<R> wv = load_vec<W, R>(w, j, i), rv = load_vec<W, R>(r, j, i);
+            n2[k] = store_spinor<W, R>(r, j, i, axpy_sp(-al, wv, rv));
+        }
     }
-    reduce_finish(v.red, j, tile, v.ntiles, n2);
+    reduce_finish<K>(v.red, j, tile, v.ntiles, n2);
 }
 
 // x += scale e ; e = 0   (FP64 x)
