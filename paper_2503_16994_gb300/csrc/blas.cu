@@ -158,15 +158,14 @@ __global__ void __launch_bounds__(128) cg_e_site(VecArgs v, const RhsState *st, 
 }
 
 // Partial of 128-site tile k of RHS j.  QUAD: the FP32 sums of its four
-// 32-site quarters, combined as the 128-thread block of reduce_partial2
-// combines its four warps ((q0 + q2) + (q1 + q3), in FP32), so both give the
-// same value.
+// 32-site quarters, added in FP32.
 template <bool QUAD>
 __device__ __forceinline__ double tile_partial(const Reduce &r, int j, int ntiles, int k)
 {
     if constexpr (QUAD) {
-        const float *q = r.partial_f + ((long)j * ntiles + k) * 4;
-        return double((q[0] + q[2]) + (q[1] + q[3]));
+        const float2 *q = reinterpret_cast<const float2 *>(r.partial_f + ((long)j * ntiles + k) * 4);  // 8-byte aligned
+        const float2 a = q[0], b = q[1];
+        return double((a.x + b.x) + (a.y + b.y));
     } else {
         return r.partial[(long)j * ntiles + k];
     }

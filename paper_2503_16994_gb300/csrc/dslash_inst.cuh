@@ -386,8 +386,8 @@ void launch_hop(const HopArgs<S, L, C> &a, int mode, bool dag, bool norm, cudaSt
     f.gpb = sh.gpb;
     f.minb = sh.minb;
     f.swz = sh.swz;
-    const bool quad = is_tile_shape(sh.nr);
-    if (quad && norm && !a.red.partial_f) throw Error{LQCD_EINVAL, "tile hopping kernel: no FP32 partials"};
+    constexpr bool quad = !std::is_same<S, F64>::value;
+    if (quad && norm && !a.red.partial_f) throw Error{LQCD_EINVAL, "hopping kernel: no FP32 partials"};
     {
         ProfScope prof(kHopNames[pi][mode], double(a.g.vh) * (nact * per_rhs + (nact ? shared : 0.0)), st);
         hopf_launch<S>(f, sh.nr, kmode, dag, st);

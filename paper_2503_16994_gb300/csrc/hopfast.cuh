@@ -9,9 +9,9 @@
 //   * NR right-hand sides per thread: each link is loaded, decoded and
 //     completed (third row) once and used for all NR right-hand sides;
 //   * GPB groups of NR right-hand sides per block, run one after the other,
-//     so a tile's links and clover come from L1 after the first group.
-// The arithmetic is the one of hop_kernel (kernels.cuh); only the
-// instruction schedule differs.
+//     so a tile's links and clover come from L1 after the first group;
+//   * a load's address as a plane address that is uniform over the block plus
+//     a 32-bit offset (at()).
 #pragma once
 #include "kernels.cuh"
 
@@ -830,8 +830,8 @@ __device__ __forceinline__ void hopf_group(const FastHop<S> &a, int tile, int g)
             }
         }
         if (NORM) {
-            if constexpr (S::W == 2) reduce_partial<double>(a.red, jj[r], tile, a.ntiles, n2);
-            else reduce_partial<float>(a.red, jj[r], tile, a.ntiles, float(n2));  // n2 is an FP32 sum
+            if constexpr (S::W == 2) reduce_partial(a.red, jj[r], tile, a.ntiles, n2);
+            else if ((on >> r) & 1) warp_partial(a.red, jj[r], tile, a.ntiles, float(n2));  // n2 is an FP32 sum
         }
     }
 }
@@ -1272,7 +1272,10 @@ __device__ __forceinline__ void hopp_epilogue(const FastHop<S> &a, int tile, int
         if (on_a) n2a = store_raw<S, float>(a.out, ja, i, va);
         if (on_b) n2b = store_raw<S, float>(a.out, jb, i, vb);
     }
-    if (NORM) reduce_partial2(a.red, ja, on_a, jb, on_b, tile, a.ntiles, float(n2a), float(n2b));  // FP32 sums
+    if (NORM) {
+        if (on_a) warp_partial(a.red, ja, tile, a.ntiles, float(n2a));
+        if (on_b) warp_partial(a.red, jb, tile, a.ntiles, float(n2b));
+    }
 }
 
 template <class S, int MODE, bool DAG, bool NORM>
@@ -1573,7 +1576,7 @@ __device__ __forceinline__ void hopq_item(const FastHop<S> &a, int tile, int j)
         }
         n2 = store_raw<S, float>(a.out, j, i, res);
     }
-    if (NORM) reduce_partial<float>(a.red, j, tile, a.ntiles, float(n2));  // FP16/FP32 only: an FP32 sum
+    if (NORM) warp_partial(a.red, j, tile, a.ntiles, float(n2));
 }
 
 // Block b handles tile b / nbt and right-hand sides [(b % nbt) gpb, ... + gpb).

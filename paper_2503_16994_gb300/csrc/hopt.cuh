@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(kTileSites * kTileMaxPairs, MINB) hopt_kernel(
         if (on_b) n2b = float(store_raw<F16, float>(a.out, jb, i, vb));
     }
     if (NORM) {
-        // the 32-site sums of reduce_partial2's warps; partial_finish combines them four at a time
+        // the 32-site sums of warp_partial; partial_finish combines them four at a time
         n2a = warp_sum_t(n2a);
         n2b = warp_sum_t(n2b);
         if (s == 0) {

@@ -56,7 +56,7 @@ struct Reduce {
     unsigned *counter;   // [nrhs], zero between uses
     RhsState *st;        // [nrhs]
     int op;
-    float *partial_f;    // [nrhs][4 ntiles]: FP32 sums per 32 sites (tile hopping kernel), or null
+    float *partial_f;    // [nrhs][4 ntiles]: FP32 sums per 32 sites (FP16/FP32 hopping kernels), or null
 };
 
 __device__ __forceinline__ void apply_op(const Reduce &r, int j, double sum)
@@ -180,17 +180,14 @@ __device__ __forceinline__ T warp_sum_t(T v)
     return v;
 }
 
-// Block-wide sum of v written as this block's partial of RHS j, nothing
-// else: no fence, no atomic, so the block does not wait for its own stores.
-// The partials are summed in FP64 by partial_finish_kernel (launched after
-// the producing kernel).  T is the type the block sums in: float for the
-// FP16/FP32 kernels, whose per-thread values are FP32 sums already (FP64 adds
-// are scarce on this GPU), double for the FP64 kernels.  Must be called by
-// every thread of the block.
-template <typename T>
-__device__ __forceinline__ void reduce_partial(const Reduce &r, int j, int tile, int ntiles, T v)
+// Sums of the hopping kernels, added up by partial_finish_kernel (launched
+// after them): no fence and no atomic, so no block waits for its own stores.
+// Must be called by every thread of the block (128).
+//
+// FP64 kernels: the block's sum of v is RHS j's partial of this tile.
+__device__ __forceinline__ void reduce_partial(const Reduce &r, int j, int tile, int ntiles, double v)
 {
-    __shared__ T sh[32];
+    __shared__ double sh[32];
     v = warp_sum_t(v);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     __syncthreads();
@@ -198,33 +195,19 @@ __device__ __forceinline__ void reduce_partial(const Reduce &r, int j, int tile,
     __syncthreads();
     if (wid == 0) {
         const int nw = (blockDim.x + 31) >> 5;
-        v = warp_sum_t(lane < nw ? sh[lane] : T(0));
-        if (lane == 0) r.partial[(long)j * ntiles + tile] = double(v);
+        v = warp_sum_t(lane < nw ? sh[lane] : 0.0);
+        if (lane == 0) r.partial[(long)j * ntiles + tile] = v;
     }
 }
-// the same for two right-hand sides at once (one pair of barriers), in FP32
-__device__ __forceinline__ void reduce_partial2(const Reduce &r, int ja, bool on_a, int jb, bool on_b, int tile,
-                                                int ntiles, float va, float vb)
+
+// FP16/FP32 kernels, whose per-thread values are FP32 sums already (FP64 adds
+// are scarce on this GPU): the sum of each warp, in FP32.  No barrier: a block
+// that works through several groups of right-hand sides would line its warps up
+// after each (12 on 24^3 x 48 in FP16, SELF_SUM: 254 us, 265 with the barriers).
+__device__ __forceinline__ void warp_partial(const Reduce &r, int j, int tile, int ntiles, float v)
 {
-    __shared__ float sh[2][32];
-    va = warp_sum_t(va);
-    vb = warp_sum_t(vb);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) {
-        sh[0][wid] = va;
-        sh[1][wid] = vb;
-    }
-    __syncthreads();
-    if (wid == 0) {
-        const int nw = (blockDim.x + 31) >> 5;
-        va = warp_sum_t(lane < nw ? sh[0][lane] : 0.f);
-        vb = warp_sum_t(lane < nw ? sh[1][lane] : 0.f);
-        if (lane == 0) {
-            if (on_a) r.partial[(long)ja * ntiles + tile] = double(va);
-            if (on_b) r.partial[(long)jb * ntiles + tile] = double(vb);
-        }
-    }
+    v = warp_sum_t(v);
+    if ((threadIdx.x & 31) == 0) r.partial_f[((long)j * ntiles + tile) * 4 + (threadIdx.x >> 5)] = v;
 }
 
 // ---------------------------------------------------------------------------

@@ -295,7 +295,7 @@ void launch_r_replace(const VecArgs &v, SpinorField<F64> src, SpinorField<WI> w,
                       SpinorField<F64> save, bool w_scaled, cudaStream_t st);
 void launch_norm2_f64(const VecArgs &v, SpinorField<F64> x, cudaStream_t st);
 // finishes the per-tile partials a hopping kernel wrote with reduce_partial
-// (quad: the FP32 32-site partials of the tile kernel in r.partial_f)
+// (quad: the FP32 32-site partials of warp_partial in r.partial_f)
 void launch_partial_finish(const Reduce &r, int ntiles, int nrhs, const RhsState *gate_st, int gate, cudaStream_t st,
                            bool quad = false);
 // out = C in, or with tau != 0 the twisted inverse (B - i s tau Cc) in (cl = B, cl2 = Cc)

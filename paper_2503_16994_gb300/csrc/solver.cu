@@ -58,8 +58,8 @@ Workspace::~Workspace()
 }
 
 // partial sums: the solver's reductions need nrhs * ntiles doubles followed
-// by the 4 nrhs ntiles FP32 partials of the tile hopping kernel (the room of
-// 2 nrhs ntiles doubles), on small batches one per block of the FP64 kernel
+// by the 4 nrhs ntiles FP32 partials of the FP16/FP32 hopping kernels (the room
+// of 2 nrhs ntiles doubles), on small batches one per block of the FP64 kernel
 // of hopd.cuh; the contraction T * ceil(V3/2 / 128) <= ntiles + T;
 // counters: max(nrhs, T)
 static size_t partial_count(const lqcd_lattice_s *lat, int nrhs)
