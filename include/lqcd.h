@@ -103,8 +103,7 @@ typedef struct lqcd_server_s *lqcd_server;   /* opaque serving loop */
  * every call takes it (0: the Wilson-clover operator).  Per chirality block
  * A_s (s = +1 spins 0-1, -1 spins 2-3) the site term A_s + i s tau, tau =
  * 2 kappa mu, is inverted as B_s - i s tau C_s with C_s = (A_s^2 + tau^2)^-1
- * and B_s = A_s C_s.  Solves at mu != 0 run on the generic (untuned) hopping
- * kernel in every storage format.  mu must be finite (LQCD_EINVAL).
+ * and B_s = A_s C_s.  mu must be finite (LQCD_EINVAL).
  * bc: LQCD_BC_PERIODIC (0), LQCD_BC_OPEN or LQCD_BC_SF; cF: the boundary
  * improvement coefficient of DiracParam (Sec. 3.3, c~_t), used with LQCD_BC_OPEN
  * and LQCD_BC_SF only (for LQCD_BC_OPEN the T
