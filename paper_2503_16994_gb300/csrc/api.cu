@@ -3,6 +3,7 @@
 // a thread-local message.
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <cstring>
 #include <new>
 #include <string>
@@ -34,6 +35,13 @@ struct DeviceGuard {
         if (prev >= 0) cudaSetDevice(prev);
     }
 };
+
+// do two arrays of the same size share bytes?
+static bool overlap(const void *a, const void *b, size_t bytes)
+{
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x < y + bytes && y < x + bytes;
+}
 
 static int check_params(const lqcd_dirac_params *dp)
 {
@@ -321,6 +329,11 @@ int lqcd_dirac_apply(lqcd_lattice lat, int gauge_id, const lqcd_dirac_params *dp
         LQCD_CUDA(cudaMemcpyAsync(lat->staging.p, psi_in, bytes, cudaMemcpyHostToDevice, st));
         in = lat->staging.as<const double>();
         out = lat->staging2.as<double>();
+    } else if (overlap(in, out, bytes)) {
+        // in place, or overlapping: the kernel reads neighbours of the sites it writes
+        lat->staging.ensure(bytes);
+        LQCD_CUDA(cudaMemcpyAsync(lat->staging.p, in, bytes, cudaMemcpyDeviceToDevice, st));
+        in = lat->staging.as<const double>();
     }
     dirac_apply_dev(lat, *it->second, *dp, in, out, (flags & LQCD_DAG) != 0, st);
     if (!(flags & LQCD_DEVICE_PTRS)) LQCD_CUDA(cudaMemcpyAsync(psi_out, out, bytes, cudaMemcpyDeviceToHost, st));

@@ -81,3 +81,25 @@ def test_solve_reports_the_true_residual(lq, dims, mu):
         r = b[j] - oracle.dirac_tm(dims, U, 0.125, 1.3, mu, x[j], theta=THETA)
         assert np.linalg.norm(r) <= 1e-12 * np.linalg.norm(b[j])
         assert abs(info[j]["true_resid"] - np.linalg.norm(r) / np.linalg.norm(b[j])) <= 1e-14
+
+
+@pytest.mark.parametrize("dims", [(4, 4, 4, 4), (8, 12, 10, 26)])
+def test_dirac_in_place(lq, dims):
+    """D reads the host layout directly; a field that it also writes is copied first."""
+    import torch
+    U = inputs.gauge_field(dims, 0.4, seed=101)
+    psi = torch.from_numpy(inputs.spinor_field(dims, seed=102)).cuda()
+    n = psi.numel()
+    lat = lq.lattice_create(dims)
+    try:
+        gid = lq.gauge_upload(lat, U)
+        dp = lq.dirac_params(0.13, 1.5)
+        want = lq.dirac_apply(lat, gid, dp, psi)
+        for shift in (0, 12 * 7):  # the same array, and one that begins seven sites later
+            room = torch.zeros(n + shift, dtype=psi.dtype, device="cuda")
+            room[:n] = psi.reshape(-1)
+            torch.cuda.synchronize()
+            got = lq.dirac_apply(lat, gid, dp, room[:n].view(psi.shape), out=room[shift:].view(psi.shape))
+            assert torch.equal(got, want)
+    finally:
+        lq.lattice_destroy(lat)
