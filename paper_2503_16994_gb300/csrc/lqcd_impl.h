@@ -194,9 +194,9 @@ template <class S> constexpr const char *prec_name() { return S::W == 2 ? "f64" 
 // become resident while the last blocks of the kernel before it on the stream
 // are still running, and wait there for its end, so the launch and the ramp-up
 // are hidden.  Used for the FP64 kernels of small batches and the reductions,
-// which take microseconds: a CG iteration of one FP64 right-hand side on 4^4
-// takes 52 us instead of 60.  The kernels of large batches gain nothing from
-// it and lose 3% by the plain loads it asks for.
+// which take microseconds: it saves 8 us of a CG iteration of one FP64
+// right-hand side on 4^4, 55 us now.  The kernels of large batches gain nothing
+// from it and lose 3% by the plain loads it asks for.
 template <typename... P, typename... A>
 inline void launch_pdl(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, A... args)
 {

@@ -400,10 +400,10 @@ struct Solver {
 
     // What the states ask for (host view after a poll): x += A_ee^-1 e for
     // the RHS whose recursion has converged, whose FP64 check is that of
-    // finish(), so the two FP64 hops of a last update are saved (a propagator
-    // on 24^3 x 48 in FP16 565 ms instead of 580, on 16^3 x 32 in FP32 91
-    // instead of 96, one FP64 column on 4^4 2.08 instead of 2.22); and the
-    // cheapest residual recomputation that the others allow.
+    // finish(), so the two FP64 hops of a last update are saved (15 ms of a
+    // propagator on 24^3 x 48 in FP16, 4.5 of one on 16^3 x 32 in FP32, 0.14 of
+    // one FP64 column on 4^4); and the cheapest residual recomputation that the
+    // others allow.
     void update_best()
     {
         if (any_status(ST_FINAL)) {
