@@ -386,7 +386,7 @@ void launch_hop(const HopArgs<S, L, C> &a, int mode, bool dag, bool norm, cudaSt
     f.gpb = sh.gpb;
     f.minb = sh.minb;
     f.swz = sh.swz;
-    constexpr bool quad = !std::is_same<S, F64>::value;
+    const bool quad = !std::is_same<S, F64>::value && kmode < TWIST;  // the sums of 32 sites in FP32 (kernels.cuh)
     if (quad && norm && !a.red.partial_f) throw Error{LQCD_EINVAL, "hopping kernel: no FP32 partials"};
     {
         ProfScope prof(kHopNames[pi][mode], double(a.g.vh) * (nact * per_rhs + (nact ? shared : 0.0)), st);

@@ -831,6 +831,7 @@ __device__ __forceinline__ void hopf_group(const FastHop<S> &a, int tile, int g)
         }
         if (NORM) {
             if constexpr (S::W == 2) reduce_partial(a.red, jj[r], tile, a.ntiles, n2);
+            else if constexpr (TW) block_partial(a.red, jj[r], tile, a.ntiles, n2);
             else if ((on >> r) & 1) warp_partial(a.red, jj[r], tile, a.ntiles, float(n2));  // n2 is an FP32 sum
         }
     }
@@ -1273,8 +1274,13 @@ __device__ __forceinline__ void hopp_epilogue(const FastHop<S> &a, int tile, int
         if (on_b) n2b = store_raw<S, float>(a.out, jb, i, vb);
     }
     if (NORM) {
-        if (on_a) warp_partial(a.red, ja, tile, a.ntiles, float(n2a));
-        if (on_b) warp_partial(a.red, jb, tile, a.ntiles, float(n2b));
+        if constexpr (TW) {
+            if (on_a) block_partial(a.red, ja, tile, a.ntiles, n2a);
+            if (on_b) block_partial(a.red, jb, tile, a.ntiles, n2b);
+        } else {
+            if (on_a) warp_partial(a.red, ja, tile, a.ntiles, float(n2a));
+            if (on_b) warp_partial(a.red, jb, tile, a.ntiles, float(n2b));
+        }
     }
 }
 

@@ -210,6 +210,16 @@ __device__ __forceinline__ void warp_partial(const Reduce &r, int j, int tile, i
     if ((threadIdx.x & 31) == 0) r.partial_f[((long)j * ntiles + tile) * 4 + (threadIdx.x >> 5)] = v;
 }
 
+// Twisted mass in FP16/FP32: the threads' values are added in FP64 from the
+// first addition on (a sum over 128 sites also leaves the range of FP32 where no
+// site does), one partial per tile.  Must be called by every thread of the block.
+__device__ __forceinline__ void block_partial(const Reduce &r, int j, int tile, int ntiles, double v)
+{
+    __shared__ double sh[128];
+    const double s = block_sum4(v, sh);
+    if (threadIdx.x == 0) r.partial[(long)j * ntiles + tile] = s;
+}
+
 // ---------------------------------------------------------------------------
 // hopping term with fused epilogues
 //
