@@ -135,9 +135,9 @@ typedef struct {
 } lqcd_solver_params;
 
 /* Per right-hand-side result.  iters_inner: normal-operator applications;
- * iters_outer: FP64 residual recomputations (reliable updates); true_resid:
- * final |b - D x| / |b| computed in FP64 on the full lattice; status: LQCD_OK
- * or LQCD_ENOCONV. */
+ * iters_outer: FP64 residual recomputations (reliable updates, the one that
+ * closes the solve among them); true_resid: final |b - D x| / |b| computed in
+ * FP64 on the full lattice; status: LQCD_OK or LQCD_ENOCONV. */
 typedef struct {
     int iters_inner;
     int iters_outer;

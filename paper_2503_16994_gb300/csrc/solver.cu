@@ -175,6 +175,7 @@ __global__ void status_change_kernel(RhsState *s, int nrhs, int from, int to)
     if (j < nrhs && s[j].status == from) {
         s[j].status = to;
         s[j].alpha = s[j].alpha_f = 0.f;  // alpha p is in e (cg_e_site)
+        if (from == ST_FINAL) s[j].updates += 1;  // its FP64 residual is that of finish()
     }
 }
 
