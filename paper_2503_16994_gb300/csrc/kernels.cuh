@@ -18,7 +18,7 @@ namespace lqcd {
 enum RhsStatus : int {
     ST_DONE = 0, ST_ACTIVE = 1, ST_UPDATE = 2, ST_MAXITER = 3, ST_IDLE = 4, ST_RESUME = 5, ST_FINAL = 6
 };
-enum RhsTrust : int { TRUST_NONE = 0, TRUST_OPEN = 1, TRUST_USED = 2 };
+enum RhsTrust : int { TRUST_NONE = 0, TRUST_OPEN = 1, TRUST_USED = 2, TRUST_MISSED = 3 };
 
 struct RhsState {
     double gamma;    // |z|^2, z = Dhat^dag r (CGLS)
@@ -36,7 +36,8 @@ struct RhsState {
     int updates;
     int maxiter;
     int resume;      // status after an FP64 residual that did not finish: ST_ACTIVE or ST_RESUME
-    int trust;       // TRUST_OPEN: a converged recursion goes to ST_FINAL instead of ST_UPDATE
+    int trust;       // TRUST_OPEN: a converged recursion goes to ST_FINAL instead of ST_UPDATE (then TRUST_USED,
+                     // and TRUST_MISSED once FP64 has not confirmed it)
     float alpha_f, beta_f;  // alpha, beta in FP32 (the FP16/FP32 vector kernels; converted once)
 };
 

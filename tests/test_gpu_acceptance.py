@@ -1,0 +1,48 @@
+"""A solve closed by its recursion meets the acceptance of one closed by an FP64 update.
+
+An FP64 residual update stops a right-hand side at tol / 2.  A recursion that
+says so has to be borne out by the FP64 residual of the full lattice at that
+same line, whatever inner_tol lets the recursion drift by; the two residuals
+agree to FP64 rounding (1e-14 of b).  Alone and batched.
+"""
+import numpy as np
+import pytest
+
+from paper_2503_16994_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lq():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2503_16994_gb300 import lqcd
+    return lqcd
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "fp16"])
+@pytest.mark.parametrize("inner", [0.0, 1e-2, 1e-3])
+def test_residuals(lq, prec, inner):
+    dims = (8, 8, 8, 12)
+    lat = lq.lattice_create(dims)
+    got = []
+    try:
+        gid = lq.gauge_upload(lat, inputs.gauge_field(dims, 0.35, seed=11))
+        for seed in range(3):
+            b = inputs.spinor_field(dims, seed=50 + seed, nrhs=8)
+            for tol in (1e-6, 3e-8, 1e-10):
+                _, info, rc = lq.cg_solve(lat, gid, lq.dirac_params(0.128, 1.4),
+                                          lq.solver_params(tol=tol, precision=prec, inner_tol=inner), b, nrhs=8)
+                assert rc == lq.OK, info
+                got += [i["true_resid"] - 0.5 * tol for i in info]
+        jobs = [(lat, gid, lq.dirac_params(k, 1.4), (0, 1, 2, 3), 12) for k in (0.12, 0.128)]
+        _, infos, _, rc = lq.pion_corr_batch(jobs, lq.solver_params(tol=1e-8, precision=prec, inner_tol=inner))
+        assert rc == lq.OK
+        got += [i["true_resid"] - 0.5e-8 for info in infos for i in info]
+    finally:
+        lq.lattice_destroy(lat)
+    assert max(got) <= 1e-14
