@@ -936,6 +936,10 @@ template <class W, class E>
 static int batch_t(lqcd_pion_job *jobs, int n, const lqcd_solver_params &sp, int chunk, cudaStream_t origin)
 {
     std::vector<std::unique_ptr<BatchJob<W, E>>> J;
+    // Jobs on one gauge field share its clover fields and SF links, which the
+    // first to need them builds on its own stream: each job waits for the ones
+    // before it (after its own builds, so those still overlap).
+    std::map<const GaugeSet *, cudaEvent_t> built;
     for (int k = 0; k < n; ++k) {
         auto b = std::make_unique<BatchJob<W, E>>();
         b->job = &jobs[k];
@@ -946,6 +950,10 @@ static int batch_t(lqcd_pion_job *jobs, int n, const lqcd_solver_params &sp, int
         if (it == b->lat->gauges.end()) throw Error{LQCD_EINVAL, "unknown gauge id in batch job " + std::to_string(k)};
         GaugeSet &g = *it->second;
         CloverSet &cl = clover_get(b->lat, g, jobs[k].dp, b->st);
+        const auto prev = built.find(&g);
+        if (prev != built.end()) LQCD_CUDA(cudaStreamWaitEvent(b->st, prev->second, 0));
+        LQCD_CUDA(cudaEventRecord(b->join, b->st));
+        built[&g] = b->join;
         b->ws = workspace_build(b->lat, 12, sp.precision, b->st, false);
         b->s = std::make_unique<Solver<W, E>>(b->lat, *b->ws, g, cl, jobs[k].dp, 12, b->st);
         point_sources(b->lat, jobs[k].src, b->s->b_e, b->s->b_o, b->st);
