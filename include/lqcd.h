@@ -207,7 +207,8 @@ int lqcd_schur_apply(lqcd_lattice lat, int gauge_id, const lqcd_dirac_params *dp
  * equations of the even-odd preconditioned (Schur) operator
  *   Dhat = A_ee - kappa^2 H_eo A_oo^-1 H_oe
  * (A = clover site term, H = hopping term) with its even site term divided out
- * on the right (Dhat A_ee^-1, for A_ee x_e), with FP64 residual recomputation
+ * on the right (Dhat A_ee^-1, for A_ee x_e; not where an entry of A_ee^-1 exceeds
+ * 8: only the odd sites' blocks have to be invertible), with FP64 residual recomputation
  * (reliable updates) and an FP64 final true-residual check on the full
  * lattice.  b, x: nrhs * 24 V doubles, host layout; host memory, or device
  * memory when flags has LQCD_DEVICE_PTRS.  x on input: with LQCD_GUESS in

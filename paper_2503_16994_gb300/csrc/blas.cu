@@ -52,7 +52,8 @@ __device__ __forceinline__ void site_inverse(const CloverField<C> &cl, const Clo
 // on 24^3 x 48 in FP16 240 us, 6.8 TB/s, and 101 for r, where p and z took 152 us
 // (5.7 TB/s) and r with e 239; one right-hand side on 32^3 x 64 82 + 39 us,
 // before 53 + 92.  (The clover words loaded after the vectors cost 18 us more.)
-template <class W, class E>
+// SITE false, here and below: CG on Dhat itself (Solver::divided), without the site blocks.
+template <class W, class E, bool SITE>
 __global__ void __launch_bounds__(128) cg_p_update(VecArgs v, const RhsState *st, SpinorField<W> z, SpinorField<W> p,
                                                    SpinorField<E> e, CloverField<W> cl, CloverField<W> cl2,
                                                    double tau)
@@ -66,7 +67,7 @@ __global__ void __launch_bounds__(128) cg_p_update(VecArgs v, const RhsState *st
     R x[24], y[24];
     // FP16: the clover words are on their way with the vectors (36 registers)
     uint4 cw[W::W == 8 ? 9 : 1];
-    if constexpr (W::W == 8) {
+    if constexpr (SITE && W::W == 8) {
 #pragma unroll
         for (int k = 0; k < 9; ++k) cw[k] = __ldg(cl.p + k * cl.stride + i);
     }
@@ -79,7 +80,8 @@ __global__ void __launch_bounds__(128) cg_p_update(VecArgs v, const RhsState *st
 #pragma unroll
     for (int q = 0; q < 24; ++q) x[q] = fma(be, x[q], y[q]);
     store_raw<W, R>(p, j, i, x);
-    if constexpr (W::W == 8) {
+    if constexpr (!SITE) return;
+    if constexpr (SITE && W::W == 8) {
         if (tau == 0.0) {
             float A[36];
 #pragma unroll
@@ -104,6 +106,7 @@ __global__ void __launch_bounds__(128) cg_p_update(VecArgs v, const RhsState *st
 // The same in FP64, a thread per (site, chirality block) in blocks of one warp:
 // the site blocks are 264 FP64 instructions, and on a small lattice a block of
 // 128 sites with all of them kept one SM busy for 8 us.
+template <bool SITE>
 __global__ void __launch_bounds__(32) cg_p_update64(VecArgs v, const RhsState *st, SpinorField<F64> z,
                                                     SpinorField<F64> p, SpinorField<F64> e, CloverField<F64> cl,
                                                     CloverField<F64> cl2, double tau)
@@ -124,6 +127,7 @@ __global__ void __launch_bounds__(32) cg_p_update64(VecArgs v, const RhsState *s
         x[2 * k + 1] = fma(be, a.y, b.y);
         pb[k * p.stride] = make_double2(x[2 * k], x[2 * k + 1]);
     }
+    if constexpr (!SITE) return;
     load_clov_block<F64, double>(cl, 0, i, blk, A);
     clov6(A, x, y);
     if (tau != 0.0) {
@@ -138,7 +142,7 @@ __global__ void __launch_bounds__(32) cg_p_update64(VecArgs v, const RhsState *s
 
 // e = A_ee^-1 (e + alpha p), the correction in terms of the solution, with the
 // step that cg_p_update would have added next (residual updates)
-template <class W, class E>
+template <class W, class E, bool SITE>
 __global__ void __launch_bounds__(128) cg_e_site(VecArgs v, const RhsState *st, SpinorField<W> p, SpinorField<E> e,
                                                  CloverField<E> cl, CloverField<E> cl2, double tau)
 {
@@ -153,8 +157,55 @@ __global__ void __launch_bounds__(128) cg_e_site(VecArgs v, const RhsState *st, 
     const R al = alpha_of<R>(st[j]);
 #pragma unroll
     for (int q = 0; q < 24; ++q) x[q] = fma(al, y[q], x[q]);
-    site_inverse<E, R>(cl, cl2, R(tau), i, x, y);
-    store_raw<E, R>(e, j, i, y);
+    if constexpr (SITE) {
+        site_inverse<E, R>(cl, cl2, R(tau), i, x, y);
+        store_raw<E, R>(e, j, i, y);
+    } else {
+        store_raw<E, R>(e, j, i, x);
+    }
+}
+
+// |x|^2 of the gated-in right-hand sides (CG on Dhat itself, whose hops have no norm of their own)
+template <class W>
+__global__ void __launch_bounds__(128) norm2_vec(VecArgs v, SpinorField<W> x)
+{
+    const int j = blockIdx.x % v.nrhs, tile = blockIdx.x / v.nrhs;
+    if (v.gate_st && v.gate_st[j].status != v.gate) return;
+    const int i = tile * blockDim.x + threadIdx.x;
+    using R = typename real_of<W>::type;
+    R t = R(0);
+    if (i < v.vh) {
+        R a[24];
+        load_scaled<W, R>(x, j, i, a);
+#pragma unroll
+        for (int q = 0; q < 24; ++q) t = fma(a[q], a[q], t);
+    }
+    reduce_finish(v.red, j, tile, v.ntiles, double(t));
+}
+
+// *out = max(*out, the bits of the largest |entry| of A_ee^-1 in FP32), which
+// order as the values do, infinities and NaN on top; twisted: of its parts B
+// and tau C.  One pass over the FP64 blocks of the even sites per clover field.
+__global__ void __launch_bounds__(128) site_inverse_max_kernel(int vh, CloverField<F64> cl, CloverField<F64> cl2,
+                                                               double tau, unsigned *out)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned m = 0;
+    if (i < vh) {
+        auto take = [&](double x) { m = max(m, __float_as_uint(fabsf(float(x)))); };
+        for (int k = 0; k < 36; ++k) {
+            const double2 w = cl.p[k * cl.stride + i];
+            take(w.x);
+            take(w.y);
+            if (tau != 0.0) {
+                const double2 c = cl2.p[k * cl2.stride + i];
+                take(tau * c.x);
+                take(tau * c.y);
+            }
+        }
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) atomicMax(out, m);
 }
 
 // Partial of 128-site tile k of RHS j.  QUAD: the FP32 sums of its four
@@ -242,15 +293,18 @@ template <class W, class E>
 void launch_p_update(const VecArgs &v, const RhsState *s, SpinorField<W> z, SpinorField<W> p, SpinorField<E> e,
                      CloverField<W> cl, CloverField<W> cl2, double tau, cudaStream_t st)
 {
+    const bool site = cl.p != nullptr;
     ProfScope prof("cg_p_update",
-                   double(v.vh) * (nact(v) * (4.0 * spinor_bytes<W>() + 2.0 * spinor_bytes<E>()) +
-                                   (tau != 0.0 ? 2.0 : 1.0) * clover_bytes<W>()),
+                   double(v.vh) * (nact(v) * ((site ? 4.0 : 3.0) * spinor_bytes<W>() + 2.0 * spinor_bytes<E>()) +
+                                   (site ? (tau != 0.0 ? 2.0 : 1.0) : 0.0) * clover_bytes<W>()),
                    st);
     if constexpr (std::is_same<W, F64>::value)
-        launch_pdl(cg_p_update64, dim3(unsigned((v.vh + 31) / 32) * unsigned(v.nrhs), 2), 32, 0, st, v, s, z, p, e,
-                   cl, cl2, tau);
+        launch_pdl(site ? cg_p_update64<true> : cg_p_update64<false>,
+                   dim3(unsigned((v.vh + 31) / 32) * unsigned(v.nrhs), 2), 32, 0, st, v, s, z, p, e, cl, cl2, tau);
+    else if (site)
+        cg_p_update<W, E, true><<<grid_of(v), kBlock, 0, st>>>(v, s, z, p, e, cl, cl2, tau);
     else
-        cg_p_update<W, E><<<grid_of(v), kBlock, 0, st>>>(v, s, z, p, e, cl, cl2, tau);
+        cg_p_update<W, E, false><<<grid_of(v), kBlock, 0, st>>>(v, s, z, p, e, cl, cl2, tau);
     LQCD_CHECK_LAUNCH();
 }
 
@@ -258,11 +312,29 @@ template <class W, class E>
 void launch_e_site(const VecArgs &v, const RhsState *s, SpinorField<W> p, SpinorField<E> e, CloverField<E> cl,
                    CloverField<E> cl2, double tau, cudaStream_t st)
 {
+    const bool site = cl.p != nullptr;
     ProfScope prof("cg_e_site",
                    double(v.vh) * (nact(v) * (2.0 * spinor_bytes<E>() + spinor_bytes<W>()) +
-                                   (tau != 0.0 ? 2.0 : 1.0) * clover_bytes<E>()),
+                                   (site ? (tau != 0.0 ? 2.0 : 1.0) : 0.0) * clover_bytes<E>()),
                    st);
-    cg_e_site<W, E><<<grid_of(v), kBlock, 0, st>>>(v, s, p, e, cl, cl2, tau);
+    if (site) cg_e_site<W, E, true><<<grid_of(v), kBlock, 0, st>>>(v, s, p, e, cl, cl2, tau);
+    else cg_e_site<W, E, false><<<grid_of(v), kBlock, 0, st>>>(v, s, p, e, cl, cl2, tau);
+    LQCD_CHECK_LAUNCH();
+}
+
+template <class W>
+void launch_norm2(const VecArgs &v, SpinorField<W> x, cudaStream_t st)
+{
+    ProfScope prof("cg_norm2", double(v.vh) * nact(v) * spinor_bytes<W>(), st);
+    norm2_vec<W><<<grid_of(v), kBlock, 0, st>>>(v, x);
+    LQCD_CHECK_LAUNCH();
+}
+
+void launch_site_inverse_max(long vh, CloverField<F64> cl, CloverField<F64> cl2, double tau, unsigned *out,
+                             cudaStream_t st)
+{
+    ProfScope prof("site_inverse_max", double(vh) * (tau != 0.0 ? 2.0 : 1.0) * clover_bytes<F64>(), st);
+    site_inverse_max_kernel<<<unsigned(ntiles_of(vh)), kBlock, 0, st>>>(int(vh), cl, cl2, tau, out);
     LQCD_CHECK_LAUNCH();
 }
 
@@ -316,6 +388,9 @@ template void launch_convert<F64, F32>(long, int, SpinorField<F64>, SpinorField<
 template void launch_convert<F64, F16>(long, int, SpinorField<F64>, SpinorField<F16>, cudaStream_t);
 template void launch_convert<F32, F64>(long, int, SpinorField<F32>, SpinorField<F64>, cudaStream_t);
 template void launch_convert<F16, F64>(long, int, SpinorField<F16>, SpinorField<F64>, cudaStream_t);
+template void launch_norm2<F64>(const VecArgs &, SpinorField<F64>, cudaStream_t);
+template void launch_norm2<F32>(const VecArgs &, SpinorField<F32>, cudaStream_t);
+template void launch_norm2<F16>(const VecArgs &, SpinorField<F16>, cudaStream_t);
 template void launch_r_update<F64>(const VecArgs &, SpinorField<F64>, SpinorField<F64>, cudaStream_t);
 template void launch_r_update<F32>(const VecArgs &, SpinorField<F32>, SpinorField<F32>, cudaStream_t);
 template void launch_r_update<F16>(const VecArgs &, SpinorField<F16>, SpinorField<F16>, cudaStream_t);

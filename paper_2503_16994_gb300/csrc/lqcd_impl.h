@@ -93,6 +93,7 @@ struct DevBuf {
 // B = A C, both Hermitian; ainv holds B and cinv holds C.
 struct CloverSet {
     double tau = 0.0;
+    float ainv_max = -1.f;       // largest |entry| of the even sites' inverse, set by the first solve
     DevBuf a64, ainv64, cinv64;  // [parity][36 double2 planes]
     DevBuf a32, ainv32, cinv32;  // [parity][18 float4 planes]
     DevBuf a16, ainv16, cinv16;  // [parity][9 uint4 planes]
@@ -281,6 +282,7 @@ void launch_dirac(const HopArgs<F64, F64, F64> &a, const double *in, double *out
 // vector kernels (blas_*.cu)
 template <class W>
 void launch_r_update(const VecArgs &v, SpinorField<W> w, SpinorField<W> r, cudaStream_t st);
+// (cl without blocks: CG on Dhat itself, z = A_ee^-1 p and e = A_ee^-1 e fall away)
 template <class W, class E>
 void launch_p_update(const VecArgs &v, const RhsState *s, SpinorField<W> z, SpinorField<W> p, SpinorField<E> e,
                      CloverField<W> cl, CloverField<W> cl2, double tau, cudaStream_t st);
@@ -293,6 +295,12 @@ void launch_x_update(const VecArgs &v, const RhsState *s, SpinorField<E> e, Spin
 template <class W, class WI>
 void launch_r_replace(const VecArgs &v, SpinorField<F64> src, SpinorField<WI> w, SpinorField<W> r,
                       SpinorField<F64> save, bool w_scaled, cudaStream_t st);
+// |x|^2 of the gated-in right-hand sides, with v.red.op
+template <class W>
+void launch_norm2(const VecArgs &v, SpinorField<W> x, cudaStream_t st);
+// *out: raised to the bits of the largest |entry| of A_ee^-1 (FP32)
+void launch_site_inverse_max(long vh, CloverField<F64> cl, CloverField<F64> cl2, double tau, unsigned *out,
+                             cudaStream_t st);
 void launch_norm2_f64(const VecArgs &v, SpinorField<F64> x, cudaStream_t st);
 // finishes the per-tile partials a hopping kernel wrote with reduce_partial
 // (quad: the FP32 32-site partials of warp_partial in r.partial_f)

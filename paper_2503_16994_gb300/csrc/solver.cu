@@ -20,10 +20,12 @@
 // commutes with g5).  M is better conditioned than Dhat: 130 iterations
 // instead of 150 on 16^3 x 32 (kappa 0.130, c_sw 1.5) and 193 instead of 229
 // (0.132, 1.7), for one more pass over the clover blocks in the p update and
-// one less in a hop.  The inner vectors are FP64, FP32 or FP16; every time the
-// inner residual has dropped by delta (or looks converged, or the iteration
-// cap is hit) the correction is added to the FP64 solution and the residual
-// is recomputed in FP64 (reliable update), keeping p.  Mixed solvers whose
+// one less in a hop.  Where A_ee^-1 has large entries it is not divided out
+// (Solver::divided): M is Dhat there, and y is x_e.  The inner vectors are FP64,
+// FP32 or FP16; every time the inner residual has dropped by delta (or looks
+// converged, or the iteration cap is hit) the correction is added to the FP64
+// solution and the residual is recomputed in FP64 (reliable update), keeping p.
+// Mixed solvers whose
 // residual is still far from tol and from the last FP64 one instead move
 // the FP64 residual by the FP32 image of the correction (incremental update,
 // below).  Per-RHS scalars and the state machine live on the device; the host
@@ -31,6 +33,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
+#include <cstring>
 
 #include "hopd.cuh"
 #include "lqcd_impl.h"
@@ -197,10 +200,21 @@ struct Solver {
     SpinorField<E> e;
     RhsState *S;
     VecArgs v;
+    CloverSet &clover;
+    // The site term is divided out while no entry of A_ee^-1 exceeds kSiteMax
+    // (smooth to rough SU(3) fields at the usual kappa c_sw have 1.2 to 1.6).  Where
+    // one even block is nearly singular A_ee^-1 spoils what it should improve,
+    // and a singular one has no inverse at all, while Dhat does not mind.
+    // Iterations of M against Dhat in FP16 at entries of 3.3 to 3.9: 27 against 156
+    // (4^3 x 6), 136/228 (6 x 4 x 8^2), 141/144 (8^4); at 9 to 11: 172/none,
+    // 539/569, 296/218; at 250 to 320: 220/316, none/1169, 2780/300.  FP64 at 3000:
+    // 54/178, 467/437, 265/209.
+    static constexpr float kSiteMax = 8.f;
+    bool divided = true;
 
     Solver(lqcd_lattice_s *l, Workspace &w_, GaugeSet &g, CloverSet &cl, const lqcd_dirac_params &dp, int n,
            cudaStream_t s)
-        : lat(l), ws(w_), nrhs(n), kappa(dp.kappa), st(s)
+        : lat(l), ws(w_), nrhs(n), kappa(dp.kappa), st(s), clover(cl)
     {
         const long Sd = lat->stride;
         b_e = fld<F64>(ws.b_e, nullptr, Sd);
@@ -306,10 +320,36 @@ struct Solver {
         if (ws.p_sc.p) LQCD_CUDA(cudaMemsetAsync(ws.p_sc.p, 0, ws.p_sc.bytes, st));
     }
 
+    // The entries of A_ee^-1 are looked at once per clover field, by the first
+    // solve: queued here, so that the fields of several jobs are built and looked
+    // at together, and waited for by choose_operator().
+    void look_at_site_term()
+    {
+        if (clover.ainv_max >= 0.f) return;
+        unsigned *dev = ws.partial.as<unsigned>();
+        LQCD_CUDA(cudaMemsetAsync(dev, 0, sizeof(unsigned), st));
+        launch_site_inverse_max(lat->vh, ai64, ci64, h64.tau, dev, st);
+        static_assert(sizeof(RhsState) >= sizeof(float), "room in the host mirror");
+        LQCD_CUDA(cudaMemcpyAsync(ws.host_state, dev, sizeof(float), cudaMemcpyDeviceToHost, st));
+        looked = true;
+    }
+    bool looked = false;
+
+    void choose_operator()
+    {
+        if (looked) {
+            LQCD_CUDA(cudaStreamSynchronize(st));
+            std::memcpy(&clover.ainv_max, ws.host_state, sizeof(float));
+            if (!(clover.ainv_max >= 0.f)) clover.ainv_max = INFINITY;  // NaN
+            looked = false;
+        }
+        divided = clover.ainv_max <= kSiteMax;
+    }
+
     // e = A_ee^-1 (e + alpha p): the correction of x_e from that of y   [gate]
     void site_correction(int gate = ST_UPDATE)
     {
-        launch_e_site<W, E>(gated(gate, RED_STORE), S, p, e, aie, cie, h64.tau, st);
+        launch_e_site<W, E>(gated(gate, RED_STORE), S, p, e, divided ? aie : CloverField<E>{}, cie, h64.tau, st);
     }
 
     // x += scale e; rhat = bhat - Dhat x (FP64); r = rhat / scale   [gate UPDATE]
@@ -429,7 +469,7 @@ struct Solver {
         a.gate = ST_ACTIVE;
         a.nactive = hint_active;
         a.parity = 1;
-        a.in = z;
+        a.in = divided ? z : p;
         a.out = t;
         a.clov = aiw;
         a.coef = kappa;
@@ -440,7 +480,13 @@ struct Solver {
         a.out = w;
         a.coef = -kappa;
         a.red.op = RED_ALPHA;
-        launch_hop(a, SELF_SUM, false, true, st);
+        if (divided) {
+            launch_hop(a, SELF_SUM, false, true, st);
+        } else {
+            a.clov = aw;
+            launch_hop(a, SELF_CLOV, false, false, st);
+            launch_norm2<W>(gated(ST_ACTIVE, RED_ALPHA), w, st);
+        }
         launch_r_update<W>(gated(ST_ACTIVE, RED_RUPDATE), w, r, st);
     }
 
@@ -463,8 +509,14 @@ struct Solver {
         a.out = z;
         a.coef = -kappa;
         a.red.op = RED_BETA;
-        launch_hop(a, ADD_CLOV, true, true, st);
-        launch_p_update<W, E>(gated(gate, RED_STORE), S, z, p, e, aiw, ciw, hw.tau, st);
+        if (divided) {
+            launch_hop(a, ADD_CLOV, true, true, st);
+        } else {
+            a.clov = aw;
+            launch_hop(a, SELF_CLOV, true, false, st);
+            launch_norm2<W>(gated(gate, RED_BETA), z, st);
+        }
+        launch_p_update<W, E>(gated(gate, RED_STORE), S, z, p, e, divided ? aiw : CloverField<W>{}, ciw, hw.tau, st);
     }
 
     void set_resume(int v)
@@ -580,6 +632,7 @@ struct Solver {
         tol_ = sp.tol;
         if (small() && cancel) trust = TRUST_NONE;
         prepare(0.5 * tol_, delta_, sp.maxiter, guess);
+        choose_operator();  // after the set-up, whose launches then hide behind the wait
         if (guess)
             reliable_update();
         else  // from x = 0 the first residual is bhat itself (x_e holds zeros)
@@ -779,6 +832,7 @@ struct Solver {
     // returns the number of RHS that did not reach tol
     int run(const lqcd_solver_params &sp, lqcd_solve_info *info, bool guess)
     {
+        look_at_site_term();
         start(sp, guess);
         iterate(sp);
         return finish_report(sp, info);
@@ -956,10 +1010,11 @@ static int batch_t(lqcd_pion_job *jobs, int n, const lqcd_solver_params &sp, int
         built[&g] = b->join;
         b->ws = workspace_build(b->lat, 12, sp.precision, b->st, false);
         b->s = std::make_unique<Solver<W, E>>(b->lat, *b->ws, g, cl, jobs[k].dp, 12, b->st);
+        b->s->look_at_site_term();
         point_sources(b->lat, jobs[k].src, b->s->b_e, b->s->b_o, b->st);
-        b->s->start(sp);
         J.push_back(std::move(b));
     }
+    for (auto &b : J) b->s->start(sp);
     // one eager iteration per job (autotunes the kernels outside any capture)
     for (auto &b : J) {
         b->s->half1();
