@@ -170,7 +170,8 @@ __device__ __forceinline__ ah3 ah_sum(const ah3 &a, double s, const ah3 &b)
 // per link and the update took 15.4 and 22.4 ms (six instructions per complex
 // product, the exponential by 3x3 products).  It costs scratch (FlowScratch,
 // 2160 bytes a site); where the device has no room for that,
-// flow_force_kernel forms the staples (10.7 ms, and 2.3 ms for the update).
+// flow_force_kernel forms both terms per link (12.2 ms, and 2.3 ms for the
+// update), with the same bits.
 // ---------------------------------------------------------------------------
 struct FlowScratch {
     double2 *low = nullptr;  // lower staples [parity][mu][slot of nu][9 planes]
@@ -258,38 +259,50 @@ __global__ void __launch_bounds__(128) force_gather_kernel(Geom g, double2 *u64,
 }
 
 // X_mu(x) = a Z_mu(x) + b X_mu(x) for every link (b = 0: X not read), the
-// staples formed here: no scratch
+// terms formed here: no scratch.  Products and sums are those of
+// plaquette_kernel and force_gather_kernel, in their order, so that the links
+// do not depend on how much memory was free (12.2 ms on 32^4; 10.7 for the
+// staples of the link, whose result differs by rounding).
 __global__ void __launch_bounds__(64) flow_force_kernel(Geom g, LinkField<F64> U, double2 *X, double a, double b)
 {
     const long cb = long(blockIdx.x) * blockDim.x + threadIdx.x;
     const int p = blockIdx.y, mu = blockIdx.z;
     if (cb >= g.vh) return;
-    int x[4], xpm[4];
+    int x[4];
     cb_coords(g, p, int(cb), x);
-    shift(g, x, mu, +1, xpm);
     m3 S;
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) S.m[i][j] = cd{0.0, 0.0};
-    for (int nu = 0; nu < 4; ++nu) {
-        if (nu == mu) continue;
-        int xpn[4], xmn[4], xpm_mn[4];
-        shift(g, x, nu, +1, xpn);
-        shift(g, x, nu, -1, xmn);
-        shift(g, xpm, nu, -1, xpm_mn);
-        const m3 f = mm(mm(link_xy(g, U, xpm, nu, false), md(link_xy(g, U, xpn, mu, false))),
-                        md(link_xy(g, U, x, nu, false)));
-        const m3 r = mm(mm(md(link_xy(g, U, xpm_mn, nu, false)), md(link_xy(g, U, xmn, mu, false))),
-                        link_xy(g, U, xmn, nu, false));
+    for (int n = 0; n < 3; ++n) {  // lower staples, from the plaquettes at x - nu
+        const int nu = n < mu ? n : n + 1;
+        int y[4], ym[4];
+        shift(g, x, nu, -1, y);
+        shift(g, y, mu, +1, ym);
+        const m3 t = mm(md(mm(link_xy(g, U, y, mu, false), link_xy(g, U, ym, nu, false))), link_xy(g, U, y, nu, false));
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
-            for (int j = 0; j < 3; ++j) S.m[i][j] = S.m[i][j] + f.m[i][j] + r.m[i][j];
+            for (int j = 0; j < 3; ++j) S.m[i][j] = n == 0 ? t.m[i][j] : S.m[i][j] + t.m[i][j];
     }
     const m3 u = link_xy(g, U, x, mu, false);
     ah3 om = ah_zero();
     ah_add(om, u, S);
+#pragma unroll
+    for (int n = 0; n < 3; ++n) {  // P - P^dag of the plaquettes at x
+        const int nu = n < mu ? n : n + 1, c = min(mu, nu), d = max(mu, nu);
+        int xc[4], xd[4];
+        shift(g, x, c, +1, xc);
+        shift(g, x, d, +1, xd);
+        ah3 w = ah_zero();
+        ah_add(w, mm(link_xy(g, U, x, c, false), link_xy(g, U, xc, d, false)),
+               md(mm(link_xy(g, U, x, d, false), link_xy(g, U, xd, c, false))));
+        const double sg = nu > mu ? 1.0 : -1.0;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            om.d[i] = fma(sg, w.d[i], om.d[i]);
+            om.o[i].re = fma(sg, w.o[i].re, om.o[i].re);
+            om.o[i].im = fma(sg, w.o[i].im, om.o[i].im);
+        }
+    }
     force_finish(om, u, X + (long)(p * 4 + mu) * 9 * g.stride, nullptr, g.stride, cb, a, b, 0.0);
 }
 
@@ -499,7 +512,7 @@ static void force_step(lqcd_lattice_s *lat, double2 *u, double2 *X, const FlowSc
         return;
     }
     {
-        ProfScope prof(force_name, double(lat->V) * 4 * (7 * 144.0 + 144.0), st);
+        ProfScope prof("force_no_scratch", double(lat->V) * 4 * (7 * 144.0 + 144.0), st);
         flow_force_kernel<<<dim3(unsigned((lat->vh + 63) / 64), 2, 4), 64, 0, st>>>(lat->geom, U, X, a, b);
         LQCD_CHECK_LAUNCH();
     }
