@@ -169,7 +169,7 @@ __device__ __forceinline__ ah3 ah_sum(const ah3 &a, double s, const ah3 &b)
 // force_gather_kernel, which also updates the link, 3.6 ms, where the staples
 // per link and the update took 15.4 and 22.4 ms (six instructions per complex
 // product, the exponential by 3x3 products).  It costs scratch (FlowScratch,
-// 2160 bytes a site); where the device has no room for that,
+// 2160 bytes a site); where the device has no room for that (FlowWork),
 // flow_force_kernel forms both terms per link (12.2 ms, and 2.3 ms for the
 // update), with the same bits.
 // ---------------------------------------------------------------------------
@@ -473,12 +473,22 @@ __global__ void __launch_bounds__(128) gauge_unpack_kernel(Geom g, long V, const
 }
 
 // scratch of the shared-plaquette force for one call; empty (both pointers
-// null) when the device has no room for it
+// null) when the device has no room for it, or when it would take more than
+// half of what is free: other threads and processes allocate meanwhile, and the
+// scratch is a convenience.  Up to kSmallScratch that is not looked at (the
+// query takes 4 us, a flow step on 4^4 150).
+constexpr size_t kSmallScratch = size_t(64) << 20;
 struct FlowWork {
     DevBuf low, up;
     FlowScratch s;
     explicit FlowWork(long stride)
     {
+        const size_t need = FlowScratch::low_bytes(stride) + FlowScratch::up_bytes(stride);
+        if (need > kSmallScratch) {
+            size_t free_b = 0, total_b = 0;
+            LQCD_CUDA(cudaMemGetInfo(&free_b, &total_b));
+            if (need > free_b / 2) return;
+        }
         try {
             low.ensure(FlowScratch::low_bytes(stride));
             up.ensure(FlowScratch::up_bytes(stride));

@@ -1,4 +1,5 @@
-"""The flows give the same bits whether or not the device has room for the force's scratch.
+"""The flows give the same bits whether or not the device has room for the force's scratch,
+and the scratch leaves as much memory free as it takes.
 
 Each call runs with plenty of memory and again with so little that its other
 fields fit and the scratch (2160 bytes a site) does not; the profile shows
@@ -72,3 +73,25 @@ def test_same_bits(lq, kind, left):
         assert np.array_equal(a, b)
     assert "force_no_scratch" not in names[0] and "force_no_scratch" in names[1]
     assert np.max(np.abs(got[0][1] - U)) > 1e-3 or kind == "back"
+
+
+@pytest.mark.parametrize("left,scratch", [(300, False), (360, True)])
+def test_scratch_leaves_as_much_as_it_takes(lq, left, scratch):
+    """16^4: 38 MB for the accumulator, 142 of scratch: 262 and 322 MB are free when it is decided."""
+    import torch
+    dims = (16, 16, 16, 16)
+    lat = lq.lattice_create(dims)
+    hog = None
+    try:
+        gid = lq.gauge_upload(lat, inputs.gauge_field(dims, 0.4, seed=93))
+        torch.cuda.synchronize()
+        free, _ = torch.cuda.mem_get_info()
+        hog = torch.empty(free - left * MB, dtype=torch.uint8, device="cuda")
+        lq.profile_reset()
+        lq.gauge_flow(lat, gid, 0.02, 1)
+        names = set(lq.profile_read())
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+        lq.lattice_destroy(lat)
+    assert ("force_no_scratch" not in names) == scratch
