@@ -51,9 +51,11 @@ __device__ __forceinline__ ah3 load_ah(const double2 *base, long stride, long cb
 // 2^k (Cayley-Hamilton: Y^3 = c1 Y + i c0 with c1 = tr Y^2 / 2 and i c0 =
 // det Y, both from Y and Y^2).  The three coefficients come from the Horner
 // form of the degree-20 Taylor polynomial, P <- 1/n! + Y P, which costs four
-// real operations a step instead of a 3x3 product, and the k squarings act on
-// the coefficients too.  k is chosen so that |Y|_F <= 1/2, where the terms
-// left out are below 1e-25.  About 200 FP64 instructions; a Taylor polynomial
+// real operations a step instead of a 3x3 product, and up to four squarings act on
+// the coefficients too; the rest, for |s X| above 8, square the matrix: the
+// coefficients of large powers are themselves large where eigenvalues nearly
+// meet, and their rounding grows as |s X|^2 (1e-11 at 1000, 1e-13 by matrices).
+// k is chosen so that |Y|_F <= 1/2, where the terms left out are below 1e-25.  About 200 FP64 instructions; a Taylor polynomial
 // with 3x3 products took 2900, and 22.4 ms for the links of 32^4 where
 // force_gather_kernel now takes 3.6 ms for the whole update.
 constexpr int kExpDegree = 20;
@@ -119,7 +121,8 @@ __device__ __forceinline__ m3 exp_ah(const ah3 &X, double s)
         q0 = t0;
     }
     // squarings: Y^3 = c1 Y + i c0, Y^4 = c1 Y^2 + i c0 Y
-    for (int n = 0; n < k; ++n) {
+    const int kc = min(k, 4);
+    for (int n = 0; n < kc; ++n) {
         const cd p12 = 2.0 * cm0(q1, q2), p22 = cm0(q2, q2);
         cd t0 = cd{-c0 * p12.im, c0 * p12.re};
         cma(t0, q0, q0);
@@ -148,6 +151,7 @@ __device__ __forceinline__ m3 exp_ah(const ah3 &X, double s)
         cma(l, q2, cd{hh[e].re, -hh[e].im});
         E.m[j][i] = l;
     }
+    for (int n = kc; n < k; ++n) E = mm(E, E);
     return E;
 }
 
