@@ -365,7 +365,8 @@ void launch_hop(const HopArgs<S, L, C> &a, int mode, bool dag, bool norm, cudaSt
     double per_rhs = sb + (mode == RESID ? 0.0 : sb) + (mode == HOP_CLOV ? 0.0 : sb) + (mode == RESID ? sb : 0.0);
     // the twisted inverse reads two Hermitian block pairs (B and C)
     const bool twinv = a.tau != 0.0 && (mode == HOP_CLOV || mode == CLOV_SUM || mode == ADD_CLOV);
-    double shared = 8.0 * link_bytes<L>() + (mode == SELF_PLAIN || mode == SELF_SUM ? 0.0 : (twinv ? 2.0 : 1.0) * clover_bytes<C>());
+    const int blocks = mode == SELF_PLAIN || mode == SELF_SUM ? 0 : (twinv ? 2 : 1) + (mode == CLOV_SUM && norm);  // (A too)
+    const double shared = 8.0 * link_bytes<L>() + blocks * clover_bytes<C>();
     const int pi = S::W == 2 ? 0 : (S::W == 4 ? 1 : 2);
     if (!mode_built(mode, dag, norm, std::is_same<S, F64>::value))
         throw Error{LQCD_EINVAL, "hopping kernel: mode not built for this precision"};

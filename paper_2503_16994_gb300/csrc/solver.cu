@@ -278,8 +278,8 @@ struct Solver {
 
     // right-hand sides expected to pass each gate, from the last host poll
     // (launch accounting only; -1 when unknown)
-    int hint_active = -1, hint_update = -1;
-    int hint(int gate) const { return gate == ST_UPDATE ? hint_update : hint_active; }
+    int hint_active = -1, hint_update = -1, hint_final = -1;
+    int hint(int gate) const { return gate == ST_UPDATE ? hint_update : (gate == ST_FINAL ? hint_final : hint_active); }
 
     VecArgs gated(int gate, int op) const
     {
@@ -583,13 +583,15 @@ struct Solver {
         LQCD_CUDA(cudaMemcpyAsync(ws.host_state, S, sizeof(RhsState) * nrhs, cudaMemcpyDeviceToHost, st));
         LQCD_CUDA(cudaStreamSynchronize(st));
         // an RHS updated in FP64 next resumes the inner iteration (or is done)
-        int act = 0, upd = 0;
+        int act = 0, upd = 0, fin = 0;
         for (int j = 0; j < nrhs; ++j) {
             act += ws.host_state[j].status == ST_ACTIVE || ws.host_state[j].status == ST_UPDATE;
             upd += ws.host_state[j].status == ST_UPDATE;
+            fin += ws.host_state[j].status == ST_FINAL;
         }
         hint_active = act;
         hint_update = upd;
+        hint_final = fin;
     }
 
     void push_states()
