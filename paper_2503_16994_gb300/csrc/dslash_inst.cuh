@@ -244,9 +244,11 @@ static HopShape hopf_tuned(FastHop<S> f, int mode, cudaStream_t st)
                 if (gpb <= f.nrhs && (gpb == 1 || f.nrhs % gpb == 0)) cand.push_back(HopShape{-pf, gpb, 1, 1});
     HopShape best{1, 1, 1, 1};
     float best_ms = 1e30f;
-    // candidates are timed on every RHS (the caller's gate may be partial;
-    // the outputs of the fast kernels are scratch fields the launch that
-    // follows overwrites)
+    // Candidates are timed on every RHS (the caller's gate may be partial), so
+    // they overwrite the output of those gated off.  That is scratch, but for
+    // the z of ADD_CLOV, which holds A_ee^-1 p from one half iteration to the
+    // next: Solver::start() launches that mode before any z is carried, so its
+    // shape is in the table from then on.
     f.gate_st = nullptr;
     cudaEvent_t e0, e1;
     LQCD_CUDA(cudaEventCreate(&e0));

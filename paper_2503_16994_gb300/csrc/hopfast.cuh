@@ -1041,34 +1041,9 @@ __device__ __forceinline__ void link_mul_u(const float u[18], const cp h[2][3], 
     }
 }
 
-// acc += sc (1 + S g_mu) psi from g; the cases of accumulate_p with every
-// add a packed fma by the per-site scale pair (sc, or nsc = -sc)
-template <int MU, int S>
-__device__ __forceinline__ void accumulate_s(cp acc[12], const cp g[2][3], float2 sc, float2 nsc)
-{
-    const float2 ps = S > 0 ? sc : nsc, ms = S > 0 ? nsc : sc;  // S sc, -S sc
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        acc[c] = cp{p_fma(g[0][c].r, sc, acc[c].r), p_fma(g[0][c].i, sc, acc[c].i)};
-        acc[3 + c] = cp{p_fma(g[1][c].r, sc, acc[3 + c].r), p_fma(g[1][c].i, sc, acc[3 + c].i)};
-        cp &l0 = acc[6 + c], &l1 = acc[9 + c];
-        if (MU == 0) {  // lower += S (i g1, i g0)
-            l0 = cp{p_fma(g[1][c].i, ms, l0.r), p_fma(g[1][c].r, ps, l0.i)};
-            l1 = cp{p_fma(g[0][c].i, ms, l1.r), p_fma(g[0][c].r, ps, l1.i)};
-        } else if (MU == 1) {  // lower += S (g1, -g0)
-            l0 = cp{p_fma(g[1][c].r, ps, l0.r), p_fma(g[1][c].i, ps, l0.i)};
-            l1 = cp{p_fma(g[0][c].r, ms, l1.r), p_fma(g[0][c].i, ms, l1.i)};
-        } else if (MU == 2) {  // lower += S (i g0, -i g1)
-            l0 = cp{p_fma(g[0][c].i, ms, l0.r), p_fma(g[0][c].r, ps, l0.i)};
-            l1 = cp{p_fma(g[1][c].i, ps, l1.r), p_fma(g[1][c].r, ms, l1.i)};
-        } else {  // lower -= S (g0, g1)
-            l0 = cp{p_fma(g[0][c].r, ms, l0.r), p_fma(g[0][c].i, ms, l0.i)};
-            l1 = cp{p_fma(g[1][c].r, ms, l1.r), p_fma(g[1][c].i, ms, l1.i)};
-        }
-    }
-}
-
-// colour c of accumulate_s: acc += sc (1 + S g_mu) psi from (g0, g1) = g[0][c], g[1][c]
+// colour c of acc += sc (1 + S g_mu) psi from (g0, g1) = g[0][c], g[1][c]; the
+// cases of accumulate_p with every add a packed fma by the per-site scale pair
+// (sc, or nsc = -sc)
 template <int MU, int S>
 __device__ __forceinline__ void accumulate_row(cp acc[12], int c, const cp &g0, const cp &g1, float2 sc, float2 nsc)
 {
@@ -1117,7 +1092,7 @@ __device__ __forceinline__ void link_row_u(const float u[18], int a, const cp h[
 // one direction of a pair of right-hand sides from their FP16 words (wa, wb,
 // scales sa, sb) and the decoded link u; each colour row of the link product
 // is phased and accumulated as soon as it is formed (the element-wise
-// operations of link_mul_u, the phase and accumulate_s, so the same bits)
+// operations of link_mul_u, the phase and accumulate_sc, so the same bits)
 template <class S, int MU, int DIR, int SP>
 __device__ __forceinline__ void dir_words(const FastHop<S> &a, const float u[18], const __half2 wa[12],
                                           const __half2 wb[12], float sa, float sb, bool wrap, cp acc[12])

@@ -159,7 +159,7 @@ struct lqcd_lattice_s {
     std::map<std::pair<int, int>, std::unique_ptr<lqcd::Workspace>> ws;  // keyed by (nrhs, precision)
     lqcd::DevBuf staging;         // host-layout fields on the device
     lqcd::DevBuf staging2;
-    lqcd::DevBuf red_partial, red_counter, red_state;  // reductions outside the solver
+    lqcd::DevBuf red_partial, red_counter;  // reductions outside the solver
     lqcd::DevBuf tables;          // the term tables of a contraction
 };
 

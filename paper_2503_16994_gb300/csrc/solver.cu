@@ -461,7 +461,11 @@ struct Solver {
     }
 
     // w = M p (|w|^2 -> alpha); r -= alpha w   [gate ACTIVE]
-    // (z holds A_ee^-1 p from the p update)
+    // (z holds A_ee^-1 p from the p update.  In FP16 storage it is rounded to 16
+    // bits, from 16-bit blocks, like p, t and w of the iteration, while e is
+    // corrected with the FP32 blocks (aie): the recursion drifts from the
+    // residual of e by a few 2^-11 of its decade, which the residual updates
+    // take out with the rest of the storage's rounding.)
     void half1()
     {
         HopArgs<W, W, W> a = hw;
