@@ -630,6 +630,12 @@ struct Solver {
     // in x_e) and the first z, p
     void start(const lqcd_solver_params &sp, bool guess = false)
     {
+        set_up(sp, guess);
+        first_direction(guess);
+    }
+
+    void set_up(const lqcd_solver_params &sp, bool guess)
+    {
         // default reliable-update factor per inner format (measured at
         // 32^3 x 64): FP16 residuals drift, so they are refreshed every
         // decade; FP32 ones hold until 5e-3
@@ -638,11 +644,14 @@ struct Solver {
         tol_ = sp.tol;
         if (small() && cancel) trust = TRUST_NONE;
         prepare(0.5 * tol_, delta_, sp.maxiter, guess);
+        // from x = 0 the first residual is bhat itself (x_e holds zeros)
+        if (!guess) launch_r_replace<W, F64>(gated(ST_UPDATE, RED_RHAT), bhat, x_e, r, x_o, false, st);
+    }
+
+    void first_direction(bool guess)
+    {
         choose_operator();  // after the set-up, whose launches then hide behind the wait
-        if (guess)
-            reliable_update();
-        else  // from x = 0 the first residual is bhat itself (x_e holds zeros)
-            launch_r_replace<W, F64>(gated(ST_UPDATE, RED_RHAT), bhat, x_e, r, x_o, false, st);
+        if (guess) reliable_update();
         half2();
     }
 
@@ -1018,9 +1027,13 @@ static int batch_t(lqcd_pion_job *jobs, int n, const lqcd_solver_params &sp, int
         b->s = std::make_unique<Solver<W, E>>(b->lat, *b->ws, g, cl, jobs[k].dp, 12, b->st);
         b->s->look_at_site_term();
         point_sources(b->lat, jobs[k].src, b->s->b_e, b->s->b_o, b->st);
+        b->s->set_up(sp, false);
+        if (!b->s->looked) b->s->first_direction(false);
         J.push_back(std::move(b));
     }
-    for (auto &b : J) b->s->start(sp);
+    // new clover fields: waited for when the work of every job is queued
+    for (auto &b : J)
+        if (b->s->looked) b->s->first_direction(false);
     // one eager iteration per job (autotunes the kernels outside any capture)
     for (auto &b : J) {
         b->s->half1();
